@@ -222,6 +222,8 @@ struct StepCtx {
     using C = typename Prec<S>::C;
     C G, Gw[2], taum[2], itau[2], mitau[2], m[2], gx, gy;
     C dA[2][3];   // A_g(alpha_k) - w_g (GEN only; 0 for a species with alpha_k = 4/9)
+    bool body;    // a body force acts (gx or gy is not zero)
+    bool unit[2]; // tau_k = 1
     Shift<S> sh;
     // With m_k = 1 (not GEN), taum = tau and the weights of U are itau.
     __device__ __forceinline__ const C (&wU() const)[2] {
@@ -247,6 +249,7 @@ struct StepCtx {
             }
             gx = c.gx;
             gy = c.gy;
+            body = gx != 0.0f || gy != 0.0f;
         } else {
             G = (C)rd.G;
             Gw[0] = (C)rd.GwA;
@@ -257,6 +260,10 @@ struct StepCtx {
             itau[1] = (C)rd.itauB;
             gx = (C)rd.gx;
             gy = (C)rd.gy;
+            // by their bits: FP64 comparisons run on the FP64 pipe
+            body = ((__double_as_longlong(rd.gx) | __double_as_longlong(rd.gy)) << 1) != 0;
+            unit[0] = __double_as_longlong(rd.itauA) == 0x3ff0000000000000LL;
+            unit[1] = __double_as_longlong(rd.itauB) == 0x3ff0000000000000LL;
             if constexpr (GEN) {
                 mitau[0] = (C)rd.mitauA;
                 mitau[1] = (C)rd.mitauB;
@@ -284,7 +291,22 @@ struct NodeState {
     C n[2], jx[2], jy[2], ax[2], ay[2];
 };
 
-template <typename S, int W, bool G>
+// wall sum of Eq. 11 over the solid neighbours, i ascending
+template <typename C>
+__device__ __forceinline__ void wall_terms(unsigned m, C& Wx, C& Wy) {
+    using Wc = Wt<C>;
+    using A = Ar<C>;
+    if (SOL(m, 0, 1)) Wx = A::add(Wx, Wc::w1);                                // i = 1
+    if (SOL(m, 1, 0)) Wy = A::add(Wy, Wc::w1);                                // i = 2
+    if (SOL(m, 0, -1)) Wx = A::sub(Wx, Wc::w1);                               // i = 3
+    if (SOL(m, -1, 0)) Wy = A::sub(Wy, Wc::w1);                               // i = 4
+    if (SOL(m, 1, 1)) { Wx = A::add(Wx, Wc::w5); Wy = A::add(Wy, Wc::w5); }   // i = 5
+    if (SOL(m, 1, -1)) { Wx = A::sub(Wx, Wc::w5); Wy = A::add(Wy, Wc::w5); }  // i = 6
+    if (SOL(m, -1, -1)) { Wx = A::sub(Wx, Wc::w5); Wy = A::sub(Wy, Wc::w5); } // i = 7
+    if (SOL(m, -1, 1)) { Wx = A::add(Wx, Wc::w5); Wy = A::sub(Wy, Wc::w5); }  // i = 8
+}
+
+template <typename S, int W, bool G, bool FULL = false>
 __device__ __forceinline__ void node_state(const StepCtx<S, G>& cx, const typename Prec<S>::C (&fc)[2][9], unsigned m,
                                            const typename Prec<S>::C (*sd)[2][W], int s_m, int s_0, int s_p, int t,
                                            NodeState<S>& ns) {
@@ -297,18 +319,6 @@ __device__ __forceinline__ void node_state(const StepCtx<S, G>& cx, const typena
         ns.n[k] = sd[s_0][k][t];
         ns.jx[k] = A::add(A::sub(A::sub(A::add(A::sub(f[1], f[3]), f[5]), f[6]), f[7]), f[8]);
         ns.jy[k] = A::sub(A::sub(A::add(A::add(A::sub(f[2], f[4]), f[5]), f[6]), f[7]), f[8]);
-    }
-    // wall sum of Eq. 11, the same for both species
-    C Wx = C(0), Wy = C(0);
-    if (m) {
-        if (SOL(m, 0, 1)) Wx = A::add(Wx, Wc::w1);                                // i = 1
-        if (SOL(m, 1, 0)) Wy = A::add(Wy, Wc::w1);                                // i = 2
-        if (SOL(m, 0, -1)) Wx = A::sub(Wx, Wc::w1);                               // i = 3
-        if (SOL(m, -1, 0)) Wy = A::sub(Wy, Wc::w1);                               // i = 4
-        if (SOL(m, 1, 1)) { Wx = A::add(Wx, Wc::w5); Wy = A::add(Wy, Wc::w5); }   // i = 5
-        if (SOL(m, 1, -1)) { Wx = A::sub(Wx, Wc::w5); Wy = A::add(Wy, Wc::w5); }  // i = 6
-        if (SOL(m, -1, -1)) { Wx = A::sub(Wx, Wc::w5); Wy = A::sub(Wy, Wc::w5); } // i = 7
-        if (SOL(m, -1, 1)) { Wx = A::add(Wx, Wc::w5); Wy = A::sub(Wy, Wc::w5); }  // i = 8
     }
     // bulk force of Eq. 9 from the neighbour densities of the other species:
     // S = ((((w1 n1 - w1 n3) + w5 n5) - w5 n6) - w5 n7) + w5 n8 (and y)
@@ -327,8 +337,103 @@ __device__ __forceinline__ void node_state(const StepCtx<S, G>& cx, const typena
         Sy = A::fma(Wc::w5, n6, Sy);
         Sy = A::fma(-Wc::w5, n7, Sy);
         Sy = A::fma(-Wc::w5, n8, Sy);
-        ns.ax[k] = A::add(A::sub(-A::mul(cx.G, Sx), A::mul(cx.Gw[k], Wx)), cx.gx);
-        ns.ay[k] = A::add(A::sub(-A::mul(cx.G, Sy), A::mul(cx.Gw[k], Wy)), cx.gy);
+        ns.ax[k] = -A::mul(cx.G, Sx);
+        ns.ay[k] = -A::mul(cx.G, Sy);
+    }
+    // wall force of Eq. 11 next to a solid (its sum is the same for both
+    // species) and the body force where there is one.  Away from solids the
+    // wall force is a zero and subtracting it, like adding a zero body force,
+    // can change nothing but the sign of a zero acceleration, which no
+    // population depends on; the velocity output (FULL) keeps both, since it
+    // may show that sign.  20 of the step's instructions per node.
+    if (FULL || m) {
+        C Wx = C(0), Wy = C(0);
+        wall_terms<C>(m, Wx, Wy);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            ns.ax[k] = A::sub(ns.ax[k], A::mul(cx.Gw[k], Wx));
+            ns.ay[k] = A::sub(ns.ay[k], A::mul(cx.Gw[k], Wy));
+        }
+    }
+    if (FULL || cx.body) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            ns.ax[k] = A::add(ns.ax[k], cx.gx);
+            ns.ay[k] = A::add(ns.ay[k], cx.gy);
+        }
+    }
+}
+
+// Two correctly rounded FP64 quotients a / d and b / d by one reciprocal, with
+// Markstein's method (Handbook of Floating-Point Arithmetic, division with a
+// fused multiply-add): y = RN(1 / d) by Newton steps (true unless the
+// significand of d is all ones), a quotient within 1 ulp after one
+// correction, and RN(q + (a - d q) y) is then the correctly rounded quotient.
+// 18 FP64 instructions where two divisions take about 34.  Operands near the
+// ends of the exponent range, or not finite, and that significand take the
+// plain divisions; a zero numerator keeps its sign through the product.
+__device__ __forceinline__ void div2(double a, double b, double d, double& qa, double& qb) {
+    const int hd = __double2hiint(d), ha = __double2hiint(a) & 0x7fffffff, hb = __double2hiint(b) & 0x7fffffff;
+    const bool za = (ha | __double2loint(a)) == 0, zb = (hb | __double2loint(b)) == 0;
+    // d in [2^-200, 2^200), numerators in [2^-623, 2^424) or zero: no step under- or overflows
+    auto in = [](int h, int lo, int hi) { return (unsigned)(h - lo) < (unsigned)(hi - lo); };
+    const bool ones = ((hd | (int)0xfff00000u) & __double2loint(d)) == -1;
+    if (!in(hd & 0x7fffffff, 0x33700000, 0x4c700000) || ones || !(za || in(ha, 0x19000000, 0x5a700000)) ||
+        !(zb || in(hb, 0x19000000, 0x5a700000))) {
+        qa = __ddiv_rn(a, d);
+        qb = __ddiv_rn(b, d);
+        return;
+    }
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;\n" : "=d"(y) : "d"(d));
+    // each Newton step squares the relative error (about 2^-20 at first); the
+    // third one rounds a value that is exact to about 2^-105
+#pragma unroll
+    for (int i = 0; i < 3; ++i) y = __fma_rn(y, __fma_rn(-d, y, 1.0), y);
+    auto quot = [&](double n, bool zero) {
+        const double q0 = __dmul_rn(n, y);
+        const double q1 = __fma_rn(__fma_rn(-d, q0, n), y, q0);
+        const double q2 = __fma_rn(__fma_rn(-d, q1, n), y, q1);
+        return zero ? q0 : q2;
+    };
+    qa = quot(a, za);
+    qb = quot(b, zb);
+}
+// Steps 6 and 7 of the canonical (FP64) order for one species: every
+// product and sum that opposite directions share is rounded once instead of
+// twice, with the same bits: 3 (-c) = -(3 c), (-c) (-c) = c c, u_x^2 and u_y^2
+// are terms of u.u, and the rest direction's c = 0 leaves 1 - b.  unit: tau = 1,
+// where the product with 1 / tau changes nothing.  The FP64 pipe bounds the
+// FP64 step (one warp instruction in about 76 cycles per scheduler), so each
+// FP64 instruction counts: 329 per node before
+// these forms and div2, 254 with them (tau = 1; tile 64x8 of the bidirectional
+// march), 887 and 722 us per step of the 8192x160 grid.
+template <typename C, bool GEN>
+__device__ __forceinline__ void feq_relax(C ux, C uy, C xx, C yy, C b, C wn0, C wn1, C wn5, const C (&dn)[3], C itau,
+                                          bool unit, const C (&f)[9], C (&fnew)[9]) {
+    using A = Ar<C>;
+    C feq[9];
+    feq[0] = A::mul(wn0, A::sub(C(1), b));
+    const C d = A::add(ux, uy), e = A::sub(uy, ux);
+    const C cp[4] = {ux, uy, d, e}, cc[4] = {xx, yy, A::mul(d, d), A::mul(e, e)};
+    constexpr int ia[4] = {1, 2, 5, 6}, ib[4] = {3, 4, 7, 8};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const C wn = q < 2 ? wn1 : wn5;
+        const C t = A::mul(C(3), cp[q]), s = A::mul(C(4.5), cc[q]);
+        feq[ia[q]] = A::mul(wn, A::sub(A::add(s, A::add(t, C(1))), b));
+        feq[ib[q]] = A::mul(wn, A::sub(A::add(s, A::sub(C(1), t)), b));
+    }
+    if constexpr (GEN) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) feq[i] = A::add(feq[i], dn[grp(i)]);
+    }
+    if (unit) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) fnew[i] = A::sub(f[i], A::sub(f[i], feq[i]));
+    } else {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) fnew[i] = A::fma(-A::sub(f[i], feq[i]), itau, f[i]);   // Eq. 2
     }
 }
 
@@ -342,13 +447,19 @@ __device__ __forceinline__ void relax(const StepCtx<S, GEN>& cx, const typename 
     using A = Ar<C>;
     // common velocity (Eq. 8) and shifted equilibrium velocities (Eq. 7)
     const C(&wu)[2] = cx.wU();
-    const C den = A::fma(ns.n[0], wu[0], A::mul(ns.n[1], wu[1]));
-    const C numx = A::fma(ns.jx[0], wu[0], A::mul(ns.jx[1], wu[1]));
-    const C numy = A::fma(ns.jy[0], wu[0], A::mul(ns.jy[1], wu[1]));
+    C den, numx, numy;
+    if (kCanonical<C> && !GEN && cx.unit[0] && cx.unit[1]) {   // both weights are 1
+        den = A::add(ns.n[0], ns.n[1]);
+        numx = A::add(ns.jx[0], ns.jx[1]);
+        numy = A::add(ns.jy[0], ns.jy[1]);
+    } else {
+        den = A::fma(ns.n[0], wu[0], A::mul(ns.n[1], wu[1]));
+        numx = A::fma(ns.jx[0], wu[0], A::mul(ns.jx[1], wu[1]));
+        numy = A::fma(ns.jy[0], wu[0], A::mul(ns.jy[1], wu[1]));
+    }
     C Ux, Uy;
     if constexpr (kCanonical<C>) {
-        Ux = A::div(numx, den);
-        Uy = A::div(numy, den);
+        div2(numx, numy, den, Ux, Uy);
     } else {
         const C rden = __frcp_rn(den);   // one reciprocal for both components
         Ux = A::mul(numx, rden);
@@ -356,24 +467,22 @@ __device__ __forceinline__ void relax(const StepCtx<S, GEN>& cx, const typename 
     }
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-        const C ux = A::fma(cx.taum[k], ns.ax[k], Ux);
-        const C uy = A::fma(cx.taum[k], ns.ay[k], Uy);
-        const C usq = A::fma(ux, ux, A::mul(uy, uy));
+        // tau_k / m_k is 1 with the model's tau = 1, and a product with 1 is exact
+        const bool one = kCanonical<C> && !GEN && cx.unit[k];
+        const C ux = one ? A::add(ns.ax[k], Ux) : A::fma(cx.taum[k], ns.ax[k], Ux);
+        const C uy = one ? A::add(ns.ay[k], Uy) : A::fma(cx.taum[k], ns.ay[k], Uy);
+        const C xx = A::mul(ux, ux), yy = A::mul(uy, uy);
+        const C usq = kCanonical<C> ? A::add(xx, yy) : A::fma(ux, ux, yy);
         const C b = A::mul(C(1.5), usq);
         const C nk = ns.n[k];
         const C wn0 = A::mul(Wc::w0, nk), wn1 = A::mul(Wc::w1, nk), wn5 = A::mul(Wc::w5, nk);
         if constexpr (kCanonical<C>) {
-            const C cu[9] = {C(0), ux, uy, -ux, -uy, A::add(ux, uy), A::add(-ux, uy), A::sub(-ux, uy), A::sub(ux, uy)};
+            C dn[3];
+            if constexpr (GEN) {
 #pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                const C wn = i == 0 ? wn0 : (i <= 4 ? wn1 : wn5);
-                const C c = cu[i];
-                // Eqs. 3-5: wn (((1 + 3 c) + 4.5 (c c)) - b)
-                C feq = A::mul(wn, A::sub(A::fma(C(4.5), A::mul(c, c), A::fma(C(3), c, C(1))), b));
-                if constexpr (GEN) feq = A::add(feq, A::mul(cx.dA[k][grp(i)], nk));   // free alpha_k
-                const C f = fc[k][i];
-                fnew[k][i] = A::fma(-A::sub(f, feq), cx.itau[k], f);   // Eq. 2: f - (f - feq) / tau
+                for (int g = 0; g < 3; ++g) dn[g] = A::mul(cx.dA[k][g], nk);   // free alpha_k
             }
+            feq_relax<C, GEN>(ux, uy, xx, yy, b, wn0, wn1, wn5, dn, cx.itau[k], cx.unit[k], fc[k], fnew[k]);
         } else {
             // Eqs. 3-5 by opposite pairs: feq(+-c) = wn (1 + 4.5 c^2 - b) +- 3 wn c;
             // Eq. 2 as f (1 - 1/tau) + feq / tau
@@ -418,7 +527,7 @@ __device__ __forceinline__ void collide_node(const StepCtx<S, G>& cx, const type
     using C = typename Prec<S>::C;
     using A = Ar<C>;
     NodeState<S> ns;
-    node_state<S, W>(cx, fc, m, sd, s_m, s_0, s_p, t, ns);
+    node_state<S, W, G, MODE == 1>(cx, fc, m, sd, s_m, s_0, s_p, t, ns);
     if (MODE == 1) {
         C rho, px, py;
         if constexpr (G) {
@@ -636,17 +745,6 @@ __device__ __forceinline__ void collide_species(const StepCtx<S, GEN>& cx, int k
     const int kb = 1 - k;
     const C nA = sd[s_0][0][c], nB = sd[s_0][1][c];
     const C jxA = jb[0][c], jyA = jb[1][c], jxB = jb[2][c], jyB = jb[3][c];
-    C Wx = C(0), Wy = C(0);
-    if (m) {
-        if (SOL(m, 0, 1)) Wx = A::add(Wx, Wc::w1);
-        if (SOL(m, 1, 0)) Wy = A::add(Wy, Wc::w1);
-        if (SOL(m, 0, -1)) Wx = A::sub(Wx, Wc::w1);
-        if (SOL(m, -1, 0)) Wy = A::sub(Wy, Wc::w1);
-        if (SOL(m, 1, 1)) { Wx = A::add(Wx, Wc::w5); Wy = A::add(Wy, Wc::w5); }
-        if (SOL(m, 1, -1)) { Wx = A::sub(Wx, Wc::w5); Wy = A::add(Wy, Wc::w5); }
-        if (SOL(m, -1, -1)) { Wx = A::sub(Wx, Wc::w5); Wy = A::sub(Wy, Wc::w5); }
-        if (SOL(m, -1, 1)) { Wx = A::add(Wx, Wc::w5); Wy = A::sub(Wy, Wc::w5); }
-    }
     const C n1 = sd[s_0][kb][c + 1], n2 = sd[s_p][kb][c], n3 = sd[s_0][kb][c - 1], n4 = sd[s_m][kb][c],
             n5 = sd[s_p][kb][c + 1], n6 = sd[s_p][kb][c - 1], n7 = sd[s_m][kb][c - 1], n8 = sd[s_m][kb][c + 1];
     C Sx = A::fma(-Wc::w1, n3, A::mul(Wc::w1, n1));
@@ -659,16 +757,24 @@ __device__ __forceinline__ void collide_species(const StepCtx<S, GEN>& cx, int k
     Sy = A::fma(Wc::w5, n6, Sy);
     Sy = A::fma(-Wc::w5, n7, Sy);
     Sy = A::fma(-Wc::w5, n8, Sy);
-    const C ax = A::add(A::sub(-A::mul(cx.G, Sx), A::mul(cx.Gw[k], Wx)), cx.gx);
-    const C ay = A::add(A::sub(-A::mul(cx.G, Sy), A::mul(cx.Gw[k], Wy)), cx.gy);
+    C ax = -A::mul(cx.G, Sx), ay = -A::mul(cx.G, Sy);
+    if (m) {
+        C Wx = C(0), Wy = C(0);
+        wall_terms<C>(m, Wx, Wy);
+        ax = A::sub(ax, A::mul(cx.Gw[k], Wx));
+        ay = A::sub(ay, A::mul(cx.Gw[k], Wy));
+    }
+    if (cx.body) {
+        ax = A::add(ax, cx.gx);
+        ay = A::add(ay, cx.gy);
+    }
     const C(&wu)[2] = cx.wU();
     const C den = A::fma(nA, wu[0], A::mul(nB, wu[1]));
     const C numx = A::fma(jxA, wu[0], A::mul(jxB, wu[1]));
     const C numy = A::fma(jyA, wu[0], A::mul(jyB, wu[1]));
     C Ux, Uy;
     if constexpr (kCanonical<C>) {
-        Ux = A::div(numx, den);
-        Uy = A::div(numy, den);
+        div2(numx, numy, den, Ux, Uy);
     } else {
         const C rden = __frcp_rn(den);
         Ux = A::mul(numx, rden);
@@ -677,20 +783,18 @@ __device__ __forceinline__ void collide_species(const StepCtx<S, GEN>& cx, int k
     const C n = k == 0 ? nA : nB;
     const C ux = A::fma(cx.taum[k], ax, Ux);
     const C uy = A::fma(cx.taum[k], ay, Uy);
-    const C usq = A::fma(ux, ux, A::mul(uy, uy));
+    const C xx = A::mul(ux, ux), yy = A::mul(uy, uy);
+    const C usq = kCanonical<C> ? A::add(xx, yy) : A::fma(ux, ux, yy);
     const C b = A::mul(C(1.5), usq);
     const C wn0 = A::mul(Wc::w0, n), wn1 = A::mul(Wc::w1, n), wn5 = A::mul(Wc::w5, n);
     C fnew[9];
     if constexpr (kCanonical<C>) {
-        const C cu[9] = {C(0), ux, uy, -ux, -uy, A::add(ux, uy), A::add(-ux, uy), A::sub(-ux, uy), A::sub(ux, uy)};
+        C dn[3];
+        if constexpr (GEN) {
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const C wn = i == 0 ? wn0 : (i <= 4 ? wn1 : wn5);
-            const C cc = cu[i];
-            C feq = A::mul(wn, A::sub(A::fma(C(4.5), A::mul(cc, cc), A::fma(C(3), cc, C(1))), b));
-            if constexpr (GEN) feq = A::add(feq, A::mul(cx.dA[k][grp(i)], n));
-            fnew[i] = A::fma(-A::sub(f[i], feq), cx.itau[k], f[i]);
+            for (int g = 0; g < 3; ++g) dn[g] = A::mul(cx.dA[k][g], n);
         }
+        feq_relax<C, GEN>(ux, uy, xx, yy, b, wn0, wn1, wn5, dn, cx.itau[k], cx.unit[k], f, fnew);
     } else {
         const C om = C(1) - cx.itau[k], it = cx.itau[k];
         const C base = C(1) - b;
