@@ -337,7 +337,16 @@ cudaError_t issue_step(lbm_t* h, int parity, cudaStream_t s) {
         const Tile* tiles = h->d_tiles;
         int par = parity;
         void* args[] = {&runs, &tiles, &par};
-        return cudaLaunchKernel(h->jit_fn, dim3(nt), dim3(2 * W), args, 0, s);
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(nt);
+        cfg.blockDim = dim3(2 * W);
+        cfg.stream = s;
+        cudaLaunchAttribute at{};   // as the other bidirectional marches (launch_step)
+        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at.val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelExC(&cfg, h->jit_fn, args);
     }
     return dispatch_step(h, [&](auto L) { return L.step(W, h->d_runs, h->d_tiles, nt, parity, s); });
 }

@@ -92,6 +92,23 @@ template <> __device__ __forceinline__ __half ldg<__half>(const __half* p) {
     return __ushort_as_half(__ldg(reinterpret_cast<const unsigned short*>(p)));
 }
 
+// NC: through the read-only path; otherwise a plain load (buffers that other
+// CTAs of the same launch write)
+template <bool NC, typename S> __device__ __forceinline__ S ldp(const S* p) {
+    if constexpr (NC) return ldg(p);
+    else return *p;
+}
+
+// Step kernels launched with programmatic dependent launch: their CTAs may
+// start, and load what no step writes, while the step before still runs; here
+// they wait for it to be complete and visible.  The next step may start only
+// from then on, so at most two steps overlap.  The populations are then read
+// by plain loads: the read-only path may hold lines from before the wait.
+__device__ __forceinline__ void step_ready() {
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+
 // Shift w_i rho_ref,k of direction group g (0 rest, 1 axis, 2 diagonal).
 template <typename S> struct Shift {
     using C = typename Prec<S>::C;
@@ -155,8 +172,8 @@ __device__ __forceinline__ unsigned nbr_solid(const Geo& g, int xm, int xc, int 
 #define SOL(m, dy, dx) (((m) >> (((dy) + 1) * 3 + ((dx) + 1))) & 1u)
 
 // Pull of one node (step 1) and its densities (step 2).
-template <typename S>
-__device__ __forceinline__ void pull_node(const S* __restrict__ src, unsigned plane, unsigned own,
+template <typename S, bool NC = true>
+__device__ __forceinline__ void pull_node(const S* src, unsigned plane, unsigned own,
                                           unsigned oxm, unsigned oxp, unsigned orm, unsigned orp,
                                           unsigned orm_xm, unsigned orm_xp, unsigned orp_xm,
                                           unsigned orp_xp, unsigned sm, const Shift<S>& sh,
@@ -166,30 +183,30 @@ __device__ __forceinline__ void pull_node(const S* __restrict__ src, unsigned pl
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             const S* p = src + (unsigned)(k * 9) * plane;
-            f[k][0] = dec(ldg(p + own), sh.v[k][0]);
-            f[k][1] = dec(ldg(p + (1 * plane + oxm)), sh.v[k][1]);
-            f[k][2] = dec(ldg(p + (2 * plane + orm)), sh.v[k][1]);
-            f[k][3] = dec(ldg(p + (3 * plane + oxp)), sh.v[k][1]);
-            f[k][4] = dec(ldg(p + (4 * plane + orp)), sh.v[k][1]);
-            f[k][5] = dec(ldg(p + (5 * plane + orm_xm)), sh.v[k][2]);
-            f[k][6] = dec(ldg(p + (6 * plane + orm_xp)), sh.v[k][2]);
-            f[k][7] = dec(ldg(p + (7 * plane + orp_xp)), sh.v[k][2]);
-            f[k][8] = dec(ldg(p + (8 * plane + orp_xm)), sh.v[k][2]);
+            f[k][0] = dec(ldp<NC>(p + own), sh.v[k][0]);
+            f[k][1] = dec(ldp<NC>(p + (1 * plane + oxm)), sh.v[k][1]);
+            f[k][2] = dec(ldp<NC>(p + (2 * plane + orm)), sh.v[k][1]);
+            f[k][3] = dec(ldp<NC>(p + (3 * plane + oxp)), sh.v[k][1]);
+            f[k][4] = dec(ldp<NC>(p + (4 * plane + orp)), sh.v[k][1]);
+            f[k][5] = dec(ldp<NC>(p + (5 * plane + orm_xm)), sh.v[k][2]);
+            f[k][6] = dec(ldp<NC>(p + (6 * plane + orm_xp)), sh.v[k][2]);
+            f[k][7] = dec(ldp<NC>(p + (7 * plane + orp_xp)), sh.v[k][2]);
+            f[k][8] = dec(ldp<NC>(p + (8 * plane + orp_xm)), sh.v[k][2]);
         }
         return;
     }
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const S* p = src + (unsigned)(k * 9) * plane;
-        f[k][0] = dec(ldg(p + own), sh.v[k][0]);
-        f[k][1] = dec(ldg(SOL(sm, 0, -1) ? p + (3 * plane + own) : p + (1 * plane + oxm)), sh.v[k][1]);
-        f[k][2] = dec(ldg(SOL(sm, -1, 0) ? p + (4 * plane + own) : p + (2 * plane + orm)), sh.v[k][1]);
-        f[k][3] = dec(ldg(SOL(sm, 0, 1) ? p + (1 * plane + own) : p + (3 * plane + oxp)), sh.v[k][1]);
-        f[k][4] = dec(ldg(SOL(sm, 1, 0) ? p + (2 * plane + own) : p + (4 * plane + orp)), sh.v[k][1]);
-        f[k][5] = dec(ldg(SOL(sm, -1, -1) ? p + (7 * plane + own) : p + (5 * plane + orm_xm)), sh.v[k][2]);
-        f[k][6] = dec(ldg(SOL(sm, -1, 1) ? p + (8 * plane + own) : p + (6 * plane + orm_xp)), sh.v[k][2]);
-        f[k][7] = dec(ldg(SOL(sm, 1, 1) ? p + (5 * plane + own) : p + (7 * plane + orp_xp)), sh.v[k][2]);
-        f[k][8] = dec(ldg(SOL(sm, 1, -1) ? p + (6 * plane + own) : p + (8 * plane + orp_xm)), sh.v[k][2]);
+        f[k][0] = dec(ldp<NC>(p + own), sh.v[k][0]);
+        f[k][1] = dec(ldp<NC>(SOL(sm, 0, -1) ? p + (3 * plane + own) : p + (1 * plane + oxm)), sh.v[k][1]);
+        f[k][2] = dec(ldp<NC>(SOL(sm, -1, 0) ? p + (4 * plane + own) : p + (2 * plane + orm)), sh.v[k][1]);
+        f[k][3] = dec(ldp<NC>(SOL(sm, 0, 1) ? p + (1 * plane + own) : p + (3 * plane + oxp)), sh.v[k][1]);
+        f[k][4] = dec(ldp<NC>(SOL(sm, 1, 0) ? p + (2 * plane + own) : p + (4 * plane + orp)), sh.v[k][1]);
+        f[k][5] = dec(ldp<NC>(SOL(sm, -1, -1) ? p + (7 * plane + own) : p + (5 * plane + orm_xm)), sh.v[k][2]);
+        f[k][6] = dec(ldp<NC>(SOL(sm, -1, 1) ? p + (8 * plane + own) : p + (6 * plane + orm_xp)), sh.v[k][2]);
+        f[k][7] = dec(ldp<NC>(SOL(sm, 1, 1) ? p + (5 * plane + own) : p + (7 * plane + orp_xp)), sh.v[k][2]);
+        f[k][8] = dec(ldp<NC>(SOL(sm, 1, -1) ? p + (6 * plane + own) : p + (8 * plane + orp_xm)), sh.v[k][2]);
     }
 }
 
@@ -1037,10 +1054,12 @@ __device__ __forceinline__ void bar_group(int g) {
     else asm volatile("bar.sync 2, %0;\n" ::"n"(N) : "memory");
 }
 
-template <typename S, int W, bool G>
-__global__ void __launch_bounds__(2 * W, (kBidirMinBlocks<S, W>)) k_step_bidir(const RunDesc* __restrict__ runs,
-                                                                              const Tile* __restrict__ tiles,
-                                                                              int parity) {
+// One tile of the march.  `ready` is called once per thread after everything
+// that does not depend on the populations has been loaded (the chained launch
+// waits there for the tiles it reads); NC as in ldp.
+template <typename S, int W, bool G, bool NC, typename Ready>
+__device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, const Tile* __restrict__ tiles, int tile,
+                                           int parity, Ready ready) {
     using C = typename Prec<S>::C;
     // FP32 arithmetic never reads f_0 after the pull (the rest population is
     // n_k minus the moving ones), so it stages 16 populations of the collided
@@ -1055,9 +1074,12 @@ __global__ void __launch_bounds__(2 * W, (kBidirMinBlocks<S, W>)) k_step_bidir(c
     __shared__ C sd[2 * NS][2][W];      // [group * NS + step slot][species][column]
     __shared__ C ps[2][2][NP][PW];      // [group][step parity][population][column]
 
-    const Tile tl = tiles[blockIdx.x];
+    const Tile tl = tiles[tile];
     const RunDesc& rd = runs[tl.run];
-    if (!step_tile_ok(tl, rd)) return;
+    if (!step_tile_ok(tl, rd)) {
+        ready();
+        return;
+    }
 #ifdef LBM_JIT_GRID
     // compiled at run time for one grid (LBM_KERNEL_BIDIR_JIT): its sizes are
     // constants, so the plane and row offsets of the 18 loads and 18 stores
@@ -1066,6 +1088,7 @@ __global__ void __launch_bounds__(2 * W, (kBidirMinBlocks<S, W>)) k_step_bidir(c
     constexpr unsigned plane = LBM_JIT_PLANE;
     if (rd.nx != nx || rd.ny != ny || rd.pitch != pitch || rd.plane != (long long)plane) {
         if (threadIdx.x == 0 && rd.err) atomicOr(rd.err, ERR_BOUNDS);
+        ready();
         return;
     }
 #else
@@ -1073,8 +1096,8 @@ __global__ void __launch_bounds__(2 * W, (kBidirMinBlocks<S, W>)) k_step_bidir(c
     const unsigned plane = (unsigned)rd.plane;
 #endif
     const Geo geo{nx, rd.cap_x0, rd.cap_x1, rd.y_bot, rd.y_top, rd.mask};
-    const S* __restrict__ src = static_cast<const S*>(rd.buf[parity]);
-    S* __restrict__ dst = static_cast<S*>(rd.buf[parity ^ 1]);
+    const S* src = static_cast<const S*>(rd.buf[parity]);
+    S* dst = static_cast<S*>(rd.buf[parity ^ 1]);
     StepCtx<S, G> cx;
     cx.load(rd);
     const int t = threadIdx.x % W, grp_d = threadIdx.x / W;   // grp_d 0: up (U), 1: down (D)
@@ -1101,7 +1124,7 @@ __global__ void __launch_bounds__(2 * W, (kBidirMinBlocks<S, W>)) k_step_bidir(c
                 const unsigned bw = (unsigned)(q.rw * pitch), bm = (unsigned)(q.rm * pitch),
                                bp = (unsigned)(q.rp * pitch);
                 C f[2][9];
-                pull_node<S>(src, plane, bw + sc.xc, bw + sc.xm, bw + sc.xp, bm + sc.xc, bp + sc.xc, bm + sc.xm,
+                pull_node<S, NC>(src, plane, bw + sc.xc, bw + sc.xm, bw + sc.xp, bm + sc.xc, bp + sc.xc, bm + sc.xm,
                              bm + sc.xp, bp + sc.xm, bp + sc.xp, smask, cx.sh, f);
                 nA = dens9(f[0]);
                 nB = dens9(f[1]);
@@ -1117,10 +1140,78 @@ __global__ void __launch_bounds__(2 * W, (kBidirMinBlocks<S, W>)) k_step_bidir(c
         sd[slot(grp_d, k)][1][t] = nB;
     };
 
+    // Plain rows: no solid among the 3x3 neighbours of any column of the strip
+    // and no wrap in y.  They need neither the solid test nor the row and
+    // column wraps: columns -1 and nx are read from the ghost columns.  Most
+    // rows are plain; the longest run of them in this tile is [pl0, pl0 + pln).
+    int pl0 = max(1, y0 - 1), pln = max(0, min(ny - 2, y1) + 1 - pl0);
+    if (geo.mask || nx < 4) pln = 0;
+    if ((geo.cx0 <= tl.x0 + sc.ncols + 1 && geo.cx1 > tl.x0 - 2) || tl.x0 == 0 || tl.x0 + sc.ncols == nx) {
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            const int y = p ? geo.yt : geo.yb;
+            if (y < 0) continue;
+            // keep the longer side of the rows y - 1 .. y + 1
+            const int a = y - 1 - pl0, b = pl0 + pln - (y + 2);
+            if (a >= pln || b >= pln) continue;   // outside
+            if (a >= b) pln = max(a, 0);
+            else {
+                pl0 = y + 2;
+                pln = max(b, 0);
+            }
+        }
+    }
+    // byte offset of this thread's column in row 0, from LBM_COL0 columns
+    // before column 0 (idle threads of a narrow last strip repeat column x0)
+    const char* const usrc = reinterpret_cast<const char*>(src - LBM_COL0);
+    char* const udst = reinterpret_cast<char*>(dst - LBM_COL0);
+    const unsigned xo = (unsigned)((sc.dcol ? tl.x0 - 1 + t : tl.x0) + LBM_COL0) * (unsigned)sizeof(S);
+    const unsigned pitchB = (unsigned)pitch * (unsigned)sizeof(S), planeB = plane * (unsigned)sizeof(S);
+    const bool ghost = ghost_r(sc.xc, nx) | ghost_l(sc.xc, nx);
+    auto pull_plain = [&](int k, int r) {
+        // 64-bit row pointers plus multiples of the plane: one wide multiply-add
+        // per access, an immediate offset where the plane is a constant
+        const char* o = usrc + (size_t)((unsigned)r * pitchB + xo);
+        const char *om = o - pitchB, *op = o + pitchB;
+        C f[2][9];
+        auto at = [&](int q, const char* row, int dx) {
+            return ldp<NC>(reinterpret_cast<const S*>(row + (unsigned long long)planeB * (unsigned)q + dx * (int)sizeof(S)));
+        };
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk) {
+            f[kk][0] = dec(at(9 * kk + 0, o, 0), cx.sh.v[kk][0]);
+            f[kk][1] = dec(at(9 * kk + 1, o, -1), cx.sh.v[kk][1]);
+            f[kk][2] = dec(at(9 * kk + 2, om, 0), cx.sh.v[kk][1]);
+            f[kk][3] = dec(at(9 * kk + 3, o, 1), cx.sh.v[kk][1]);
+            f[kk][4] = dec(at(9 * kk + 4, op, 0), cx.sh.v[kk][1]);
+            f[kk][5] = dec(at(9 * kk + 5, om, -1), cx.sh.v[kk][2]);
+            f[kk][6] = dec(at(9 * kk + 6, om, 1), cx.sh.v[kk][2]);
+            f[kk][7] = dec(at(9 * kk + 7, op, 1), cx.sh.v[kk][2]);
+            f[kk][8] = dec(at(9 * kk + 8, op, -1), cx.sh.v[kk][2]);
+        }
+        sd[slot(grp_d, k)][0][t] = dens9(f[0]);
+        sd[slot(grp_d, k)][1][t] = dens9(f[1]);
+        if (sc.coll && k < nrows) {
+#pragma unroll
+            for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+                for (int i = kF ? 1 : 0; i < 9; ++i) ps[grp_d][k & 1][pidx(kk, i)][pc] = f[kk][i];
+        }
+    };
+
+    ready();
     unsigned sm_prev = 0, sm_cur = 0;
     for (int k = 0; k < nsteps; ++k) {
         // this group pulls rows 0 .. nrows (the last is its halo row)
-        if (k <= nrows) pull(k, sm_cur);
+        if (k <= nrows) {
+            const int r = row_at(k);
+            if ((unsigned)(r - pl0) < (unsigned)pln) {
+                pull_plain(k, r);
+                sm_cur = 0;
+            } else {
+                pull(k, sm_cur);
+            }
+        }
         if (k == 0 || (kF && k == 2))
             __syncthreads();
         else
@@ -1139,6 +1230,19 @@ __global__ void __launch_bounds__(2 * W, (kBidirMinBlocks<S, W>)) k_step_bidir(c
 #pragma unroll
                 for (int i = 0; i < 9; ++i)
                     fc[kk][i] = (kF && i == 0) ? C(0) : ps[grp_d][(k - 1) & 1][pidx(kk, i)][pc];
+            if ((unsigned)(r - pl0) < (unsigned)pln && !ghost) {
+                NodeState<S> ns;
+                node_state<S, W>(cx, fc, 0u, sd, s_m, s_row, s_p, t, ns);
+                C fn[2][9];
+                relax<S>(cx, fc, ns, fn);
+                char* o = udst + (size_t)((unsigned)r * pitchB + xo);
+#pragma unroll
+                for (int q = 0; q < 18; ++q)
+                    enc(reinterpret_cast<S*>(o + (unsigned long long)planeB * (unsigned)q), fn[q / 9][q % 9],
+                        cx.sh.v[q / 9][grp(q % 9)]);
+                sm_prev = sm_cur;
+                continue;
+            }
             const int rw = rows_of(r, ny).rw;
             collide_any<S, W, 0>(cx, fc, sm_prev, sd, s_m, s_row, s_p, t, dst, plane,
                                  (unsigned)(rw * pitch + sc.xc), MomOut{nullptr, nullptr, 0}, 0, ghost_r(sc.xc, nx),
@@ -1146,6 +1250,13 @@ __global__ void __launch_bounds__(2 * W, (kBidirMinBlocks<S, W>)) k_step_bidir(c
         }
         sm_prev = sm_cur;
     }
+}
+
+template <typename S, int W, bool G>
+__global__ void __launch_bounds__(2 * W, (kBidirMinBlocks<S, W>)) k_step_bidir(const RunDesc* __restrict__ runs,
+                                                                              const Tile* __restrict__ tiles,
+                                                                              int parity) {
+    bidir_tile<S, W, G, false>(runs, tiles, blockIdx.x, parity, [] { step_ready(); });
 }
 
 // ---- two-columns-per-thread variant ---------------------------------------------
@@ -1377,19 +1488,22 @@ __global__ void __launch_bounds__(W, (kPairMinBlocks<S, W>)) k_step_pair(const R
 template <typename S, int W, int TY>
 constexpr int kTileMinBlocks = sizeof(typename Prec<S>::C) == 8 ? 1 : 1024 / (W * TY);   // 64 registers
 
-template <typename S, int W, int TY, bool G>
-__global__ void __launch_bounds__(W * TY, (kTileMinBlocks<S, W, TY>)) k_step_tile(const RunDesc* __restrict__ runs,
-                                                                                const Tile* __restrict__ tiles,
-                                                                                int parity) {
+template <typename S, int W, int TY, bool G, bool NC, typename Ready>
+__device__ __forceinline__ void node_tile(const RunDesc* __restrict__ runs, const Tile* __restrict__ tiles, int tile,
+                                          int parity, Ready ready) {   // ready, NC: as in bidir_tile
     using C = typename Prec<S>::C;
     __shared__ C sd[TY][2][W];   // [tile row][species][tile column]
 
-    const Tile tl = tiles[blockIdx.x];
+    const Tile tl = tiles[tile];
     const RunDesc& rd = runs[tl.run];
-    if (!step_tile_ok(tl, rd)) return;
+    if (!step_tile_ok(tl, rd)) {
+        ready();
+        return;
+    }
     const int nx = rd.nx, ny = rd.ny, pitch = rd.pitch;
     const unsigned plane = (unsigned)rd.plane;
-    const S* __restrict__ src = static_cast<const S*>(rd.buf[parity]);
+    const S* src = static_cast<const S*>(rd.buf[parity]);
+    S* dst = static_cast<S*>(rd.buf[parity ^ 1]);
     const int tx = threadIdx.x % W, ty = threadIdx.x / W;
     const int x = tl.x0 - 1 + tx;                          // unwrapped column, in [-1, nx] when active
     const int r = tl.y0 - 1 + ty;                          // unwrapped row, in [-1, ny] when active
@@ -1404,11 +1518,14 @@ __global__ void __launch_bounds__(W * TY, (kTileMinBlocks<S, W, TY>)) k_step_til
     if (act) {
         const Geo geo{nx, rd.cap_x0, rd.cap_x1, rd.y_bot, rd.y_top, rd.mask};
         m = nbr_solid(geo, xw == 0 ? nx - 1 : xw - 1, xw, xw == nx - 1 ? 0 : xw + 1, q.rm, q.rw, q.rp);
+    }
+    ready();
+    if (act) {
         if (!SOL(m, 0, 0)) {
             // offsets from column -2, so that every offset is non-negative
             const unsigned bw = (unsigned)(q.rw * pitch), bm = (unsigned)(q.rm * pitch), bp = (unsigned)(q.rp * pitch);
             const unsigned xo = (unsigned)(x + 2);
-            pull_node<S>(src - 2, plane, bw + xo, bw + (xo - 1), bw + (xo + 1), bm + xo, bp + xo, bm + (xo - 1),
+            pull_node<S, NC>(src - 2, plane, bw + xo, bw + (xo - 1), bw + (xo + 1), bm + xo, bp + xo, bm + (xo - 1),
                          bm + (xo + 1), bp + (xo - 1), bp + (xo + 1), m, cx.sh, f);
             nA = dens9(f[0]);
             nB = dens9(f[1]);
@@ -1419,9 +1536,16 @@ __global__ void __launch_bounds__(W * TY, (kTileMinBlocks<S, W, TY>)) k_step_til
     __syncthreads();
     const bool coll = act && tx >= 1 && tx < W - 1 && x < nx && ty >= 1 && ty < TY - 1 && r < tl.y1;
     if (coll && !SOL(m, 0, 0))
-        collide_any<S, W, 0>(cx, f, m, sd, ty - 1, ty, ty + 1, tx, static_cast<S*>(rd.buf[parity ^ 1]), plane,
+        collide_any<S, W, 0>(cx, f, m, sd, ty - 1, ty, ty + 1, tx, dst, plane,
                              (unsigned)(q.rw * pitch + xw), MomOut{nullptr, nullptr, 0}, 0, ghost_r(xw, nx),
                              ghost_l(xw, nx));
+}
+
+template <typename S, int W, int TY, bool G>
+__global__ void __launch_bounds__(W * TY, (kTileMinBlocks<S, W, TY>)) k_step_tile(const RunDesc* __restrict__ runs,
+                                                                                const Tile* __restrict__ tiles,
+                                                                                int parity) {
+    node_tile<S, W, TY, G, false>(runs, tiles, blockIdx.x, parity, [] { step_ready(); });
 }
 
 // ---- software-pipelined staged variant ---------------------------------------

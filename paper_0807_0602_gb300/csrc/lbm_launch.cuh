@@ -24,6 +24,22 @@ static inline cudaError_t ensure_dynamic_smem(const void* fn, int bytes, std::at
     return e;
 }
 
+// Launches a step kernel so that its CTAs may start while the kernel before it
+// on the stream ends (it waits itself, step_ready).
+template <typename... P, typename... Q>
+static cudaError_t launch_step(void (*fn)(P...), int grid, int threads, cudaStream_t s, Q... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fn, P(args)...);
+}
+
 static inline int clamp_grid(long long want, int cap) {
     if (want < 1) return 1;
     return want > cap ? cap : (int)want;
@@ -193,14 +209,13 @@ cudaError_t Step<S, G>::step_tile(int W, int R, const RunDesc* d_runs, const Til
     if (ntiles <= 0) return cudaSuccess;
     // R = collided rows per tile: TY = R + 2 thread rows
     switch (W * 100 + R) {
-        case 3206: k_step_tile<S, 32, 8, G><<<ntiles, 256, 0, s>>>(d_runs, d_tiles, parity); break;
-        case 3214: k_step_tile<S, 32, 16, G><<<ntiles, 512, 0, s>>>(d_runs, d_tiles, parity); break;
-        case 3230: k_step_tile<S, 32, 32, G><<<ntiles, 1024, 0, s>>>(d_runs, d_tiles, parity); break;
-        case 6406: k_step_tile<S, 64, 8, G><<<ntiles, 512, 0, s>>>(d_runs, d_tiles, parity); break;
-        case 6414: k_step_tile<S, 64, 16, G><<<ntiles, 1024, 0, s>>>(d_runs, d_tiles, parity); break;
+        case 3206: return launch_step(k_step_tile<S, 32, 8, G>, ntiles, 256, s, d_runs, d_tiles, parity);
+        case 3214: return launch_step(k_step_tile<S, 32, 16, G>, ntiles, 512, s, d_runs, d_tiles, parity);
+        case 3230: return launch_step(k_step_tile<S, 32, 32, G>, ntiles, 1024, s, d_runs, d_tiles, parity);
+        case 6406: return launch_step(k_step_tile<S, 64, 8, G>, ntiles, 512, s, d_runs, d_tiles, parity);
+        case 6414: return launch_step(k_step_tile<S, 64, 16, G>, ntiles, 1024, s, d_runs, d_tiles, parity);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 template <typename S, bool G>
@@ -208,14 +223,12 @@ cudaError_t Step<S, G>::step_bidir(int W, const RunDesc* d_runs, const Tile* d_t
                                   cudaStream_t s) {
     if (ntiles <= 0) return cudaSuccess;
     switch (W) {
-        case 64: k_step_bidir<S, 64, G><<<ntiles, 128, 0, s>>>(d_runs, d_tiles, parity); break;
+        case 64: return launch_step(k_step_bidir<S, 64, G>, ntiles, 128, s, d_runs, d_tiles, parity);
         case 128:
             if constexpr (sizeof(typename Prec<S>::C) == 8) return cudaErrorInvalidValue;
-            else k_step_bidir<S, 128, G><<<ntiles, 256, 0, s>>>(d_runs, d_tiles, parity);
-            break;
+            else return launch_step(k_step_bidir<S, 128, G>, ntiles, 256, s, d_runs, d_tiles, parity);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 template <typename S, int D, bool G>
