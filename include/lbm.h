@@ -354,6 +354,13 @@ int lbm_set_tiling(lbm_t* h, int tile_w, int tile_h);
  *                         process; setting the schedule returns LBM_ECUDA if
  *                         the run-time compiler or the module load fails,
  *                         and the handle then keeps its previous schedule.
+ *   LBM_KERNEL_CHAIN      LBM_KERNEL_BIDIR's tiles, many steps in one launch:
+ *                         CTAs draw (step, tile) items from a device counter
+ *                         and wait for the neighbouring tiles' step before
+ *                         only (LBM_F64; tile_w 64).  lbm_step then issues
+ *                         all its steps up to the next log record as one
+ *                         launch (graph_chunk > 0: that many), inside a CUDA
+ *                         graph where the log is on and whole.
  * depth is read by LBM_KERNEL_ASYNC, LBM_KERNEL_TMA and LBM_KERNEL_RING and
  * must be 4 for the others.  lbm_set_schedule returns LBM_EINVAL for an unsupported
  * combination, leaving the schedule unchanged. */
@@ -370,6 +377,7 @@ int lbm_set_tiling(lbm_t* h, int tile_w, int tile_h);
 #define LBM_KERNEL_BIDIR 9       /* two thread groups marching away from the tile's middle row */
 #define LBM_KERNEL_RING 10       /* persistent producer/consumer ring of bulk-copied row slots (FP32, FP16S) */
 #define LBM_KERNEL_BIDIR_JIT 11  /* LBM_KERNEL_BIDIR compiled at run time for the handle's grid (one run) */
+#define LBM_KERNEL_CHAIN 12      /* LBM_KERNEL_BIDIR's tiles, many steps chained in one launch (FP64) */
 int lbm_get_schedule(const lbm_t* h, int* tile_w, int* tile_h, int* kernel, int* depth);
 /* The autotuner's finalists (the paper has no counterpart: this reports on the
  * library's own schedule search).  *count = number of finalists (0 before

@@ -55,9 +55,15 @@ struct lbm_s {
                                    // thread, 8 one node per thread over a W x (R + 2) tile, 9 two thread
                                    // groups marching away from the tile's middle row, 10 persistent
                                    // producer/consumer ring of row slots filled by bulk copies, 11 the
-                                   // bidirectional march compiled at run time for the run's grid
+                                   // bidirectional march compiled at run time for the run's grid, 12
+                                   // chained steps over bidirectional tiles (lbm_chain.cuh)
     int* d_queue = nullptr;        // ring kernel: segment counter and finished-CTA counter
     int ring_grid = 0;             // ring kernel: CTAs of the persistent grid
+    std::vector<int> chain_tab;    // chained steps (kvar 12): ChainTiles' tables, deps, flags, control words, span
+    int* d_chain = nullptr;
+    int chain_cap = 0;             // tiles these tables have room for
+    int chain_grid = 0;            // CTAs of a chained launch
+    int chain_rot = 0;             // tiles each step starts further on
     const void* jit_fn = nullptr;  // kvar 11: the bidirectional march compiled for this run's grid
     std::vector<int2> rows;
     int2* d_rows = nullptr;
@@ -239,6 +245,56 @@ void build_tiles(lbm_t* h, int W, int R) {
     }
 }
 
+// Chained steps (kvar 12): the tiles of a run down the columns of tiles, and
+// their tables (chain_tables).  A tile waits for the tiles with nodes within
+// two nodes of its own (periodic): the pull reads one node around and the
+// densities of the force one more, and a tile's stores overwrite what those
+// tiles read the step before.
+void build_chain_tiles(lbm_t* h, int W, int R) {
+    const int Wc = W - 2;
+    h->tiles.clear();
+    h->tile_begin.assign(h->nruns, 0);
+    h->tile_count.assign(h->nruns, 0);
+    h->chain_rot = 2;
+    for (int r = 0; r < h->nruns; ++r) {
+        const RunDesc& rd = h->runs[r];
+        const int Rr = std::max(1, std::min(R, rd.ny)), rows = (rd.ny + Rr - 1) / Rr;
+        h->tile_begin[r] = (int)h->tiles.size();
+        for (int x0 = 0; x0 < rd.nx; x0 += Wc)
+            for (int y0 = 0; y0 < rd.ny; y0 += Rr) h->tiles.push_back({r, x0, y0, std::min(y0 + Rr, rd.ny)});
+        h->tile_count[r] = (int)h->tiles.size() - h->tile_begin[r];
+        h->chain_rot = std::max(h->chain_rot, std::min(2 * rows, 1023));
+    }
+    const size_t nt = h->tiles.size();
+    h->chain_tab.assign(nt * (sc::kChainDeps + 3) + 4, 0);
+    int* deps = h->chain_tab.data();
+    int* span = deps + nt * sc::kChainDeps;
+    std::fill(deps, span, -1);
+    // pieces (of `size` cells of n) with cells within two of piece p
+    auto near = [](int p, int size, int n, int (&out)[5]) {
+        const int lo = p * size, hi = std::min(lo + size, n) - 1;
+        int k = 0;
+        for (int c : {lo - 2, lo - 1, lo, hi + 1, hi + 2}) {
+            const int q = (((c % n) + n) % n) / size;
+            if (std::find(out, out + k, q) == out + k) out[k++] = q;
+        }
+        return k;
+    };
+    for (int r = 0; r < h->nruns; ++r) {
+        const RunDesc& rd = h->runs[r];
+        const int t0 = h->tile_begin[r], Rr = std::max(1, std::min(R, rd.ny)), rows = (rd.ny + Rr - 1) / Rr;
+        for (int j = 0; j < h->tile_count[r]; ++j) {
+            int nc[5], nr[5];
+            const int kc = near(j / rows, Wc, rd.nx, nc), kr = near(j % rows, Rr, rd.ny, nr);
+            int* d = deps + (size_t)(t0 + j) * sc::kChainDeps;
+            for (int x = 0; x < kc; ++x)
+                for (int y = 0; y < kr; ++y) *d++ = t0 + nc[x] * rows + nr[y];   // at most 5 x 5
+            span[2 * (t0 + j)] = t0;
+            span[2 * (t0 + j) + 1] = h->tile_count[r];
+        }
+    }
+}
+
 void drop_graphs(lbm_t* h) {
     for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second);
     h->graphs.clear();
@@ -255,8 +311,43 @@ int ring_grid_size(lbm_t* h, int D, int* grid) {
     return LBM_OK;
 }
 
+// Device tables of the chained steps, in one allocation: deps and span (written
+// by the host), control words and flags (zero between launches).
+sc::ChainTiles chain_tables(const lbm_t* h) {
+    const int nt = (int)h->tiles.size();
+    int* p = h->d_chain;
+    return {h->d_tiles, reinterpret_cast<const int2*>(p + (size_t)nt * sc::kChainDeps), p,
+            p + (size_t)nt * (sc::kChainDeps + 2) + 4,
+            reinterpret_cast<sc::ChainCtl*>(p + (size_t)nt * (sc::kChainDeps + 2)), nt};
+}
+
+int upload_chain(lbm_t* h, int W, int R) {
+    build_chain_tiles(h, W, R);
+    const int nt = (int)h->tiles.size();
+    int per_sm = 0, dev = 0, sms = 0;
+    CK(h, dispatch_step(h, [&](auto L) { return L.chain_ctas_per_sm(&per_sm); }));
+    CK(h, cudaGetDevice(&dev));
+    CK(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (per_sm < 1 || sms < 1) return LBM_EINVAL;
+    h->chain_grid = std::min(per_sm * sms, 2 * nt);
+    const size_t bytes = h->chain_tab.size() * sizeof(int);
+    if (nt > h->chain_cap) {
+        // the old tables may still be in use by queued work: kept until destroy
+        int* p = static_cast<int*>(dalloc(h, bytes));
+        if (!p) return LBM_ENOMEM;
+        h->d_chain = p;
+        h->chain_cap = nt;
+    }
+    // upload_tiles synchronises before the vector can change
+    CK(h, cudaMemcpyAsync(h->d_chain, h->chain_tab.data(), bytes, cudaMemcpyHostToDevice, h->stream));
+    return LBM_OK;
+}
+
 int upload_tiles(lbm_t* h, int W, int R) {
-    if (h->kvar == 10) {
+    if (h->kvar == 12) {
+        const int rc = upload_chain(h, W, R);
+        if (rc) return rc;
+    } else if (h->kvar == 10) {
         int G = 0;
         int rc = ring_grid_size(h, h->depth, &G);
         if (rc) return rc;
@@ -302,9 +393,23 @@ sc::LogCtl logctl(lbm_t* h) {
     return lc;
 }
 
+// Issues n chained steps on stream s (parity = t & 1 of the first).
+cudaError_t issue_chain(lbm_t* h, int parity, int n, cudaStream_t s) {
+    const int nt = (int)h->tiles.size();
+    const sc::ChainTiles ct = chain_tables(h);
+    // a single step has nothing to chain: no more CTAs than tiles
+    const int grid = n == 1 ? std::min(h->chain_grid, nt) : h->chain_grid;
+    return dispatch_step(h, [&](auto L) {
+        return L.chain(h->d_runs, ct, n, parity, h->chain_rot, grid, h->d_err, s);
+    });
+}
+
+bool chained(const lbm_t* h) { return h->kvar == 12; }
+
 // Issues one time step on stream s (parity = t & 1 of the step).
 cudaError_t issue_step(lbm_t* h, int parity, cudaStream_t s) {
     const int W = h->tile_w, nt = (int)h->tiles.size();
+    if (chained(h)) return issue_chain(h, parity, 1, s);
     if (h->kvar == 1)
         return dispatch_step(h,
                              [&](auto L) { return L.step_async(W, h->depth, h->d_runs, h->d_tiles, nt, parity, s); });
@@ -352,7 +457,11 @@ cudaError_t issue_step(lbm_t* h, int parity, cudaStream_t s) {
 }
 
 bool schedule_ok(const lbm_t* h, int W, int R, int kvar, int depth) {
-    if (R < 1 || kvar < 0 || kvar > 11) return false;
+    if (R < 1 || kvar < 0 || kvar > 12) return false;
+    if (kvar == 12) {   // chained bidirectional tiles: FP64, and the march's tilings
+        if (h->precision != LBM_F64) return false;
+        kvar = 9;
+    }
     if (kvar == 11) {   // the bidirectional march compiled for the grid: one run per handle
         if (h->nruns != 1) return false;
         kvar = 9;
@@ -436,7 +545,9 @@ int get_graph(lbm_t* h, int parity, int steps, int with_log, cudaGraphExec_t* ou
     cudaGraph_t g = nullptr;
     CK(h, cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
-    for (int j = 0; j < steps && e == cudaSuccess; ++j) e = issue_step(h, (parity + j) & 1, h->cap_stream);
+    if (chained(h)) e = issue_chain(h, parity, steps, h->cap_stream);
+    else
+        for (int j = 0; j < steps && e == cudaSuccess; ++j) e = issue_step(h, (parity + j) & 1, h->cap_stream);
     if (e == cudaSuccess && with_log) e = issue_log(h, (parity + steps) & 1, h->cap_stream);
     cudaError_t e2 = cudaStreamEndCapture(h->cap_stream, &g);
     if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -471,7 +582,18 @@ int advance(lbm_t* h, int64_t n) {
         int64_t m;
         if (le > 0) m = std::min<int64_t>(n, le - (h->t % le));
         else m = std::min<int64_t>(n, chunk);
-        if (graphs && m == chunk && (le == 0 || h->t % le == 0)) {
+        if (chained(h) && (le == 0 || !graphs || m != le)) {
+            // one launch for all of them (with the log on and whole chunks: within their graph)
+            NvtxRange range("lbm chained steps");
+            const int64_t most = std::max<int64_t>(1, (1 << 30) / (int64_t)h->tiles.size());   // 32-bit item numbers
+            m = std::min(le > 0 ? m : (h->opt.graph_chunk > 0 ? m : n), most);
+            CK(h, issue_chain(h, (int)(h->t & 1), (int)m, h->stream));
+            h->t += m;
+            if (le > 0 && h->t % le == 0) {
+                CK(h, issue_log(h, (int)(h->t & 1), h->stream));
+                h->nlog += 1;
+            }
+        } else if (graphs && m == chunk && (le == 0 || h->t % le == 0)) {
             NvtxRange range("lbm graph chunk");
             cudaGraphExec_t ex;
             int rc = get_graph(h, (int)(h->t & 1), chunk, le > 0, &ex);
@@ -525,12 +647,14 @@ int wave_height(lbm_t* h, int W, int waves) {
     return lo;
 }
 
+struct Sched {
+    int W, R, kvar, depth;
+};
+
 // Times candidate tilings on the live state: the steps taken are real steps
 // (every tiling computes the same bits), only their schedule differs.
 int autotune(lbm_t* h, int64_t* n) {
-    struct Cand {
-        int W, R, kvar, depth;
-    };
+    using Cand = Sched;
     int maxny = 1;
     for (auto& rd : h->runs) maxny = std::max(maxny, rd.ny);
     std::vector<int> Rs = {4, 8, 16, 32};
@@ -574,6 +698,8 @@ int autotune(lbm_t* h, int64_t* n) {
             if (schedule_ok(h, W, R, 8, 4)) cands.push_back({W, R, 8, 4});
     for (int D : {3, 4, 5})
         if (schedule_ok(h, 128, 4, 10, D)) cands.push_back({128, 4, 10, D});
+    for (int R : {2, 4, 8, 16})
+        if (R <= maxny && schedule_ok(h, 64, R, 12, 4)) cands.push_back({64, R, 12, 4});
     // pass 1: every candidate for `per` steps; pass 2: the kFinal fastest in
     // `rounds` interleaved rounds of per_final steps each, scored by their
     // best round (candidates within a few per cent of each other are told
@@ -870,7 +996,7 @@ int fetch_fields(lbm_t* h, int run, double* a, double* b, int on_device, bool ve
         if (e == cudaSuccess) e = cudaMemsetAsync(db, 0, nn * sizeof(double), h->stream);
     } else {
         sc::MomOut mo{da, db, rd.nx};
-        const int W = h->tile_w;
+        const int W = h->kvar == 7 ? 2 * h->tile_w : h->tile_w;   // the pair kernel's tiles are 2 W - 4 columns wide
         e = dispatch_step(h, [&](auto L) {
             return L.moments(W, h->d_runs, h->d_tiles + h->tile_begin[run], h->tile_count[run], (int)((h->t - 1) & 1),
                              mo, h->stream);

@@ -94,6 +94,26 @@ struct Tile {
     int run, x0, y0, y1;
 };
 
+// Control words of a chained launch, all zero before it and after it.
+struct ChainCtl {
+    int next;      // next item
+    int done;      // CTAs that have finished
+    int abort;     // a wait gave up
+    int pad;
+};
+
+// Per tile: where its run's tiles start and how many they are.
+struct ChainTiles {
+    const Tile* tiles;
+    const int2* span;     // [ntiles] (first tile, number of tiles) of the tile's run
+    const int* deps;      // [ntiles][kChainDeps] tiles to wait for, -1 = none
+    int* flags;           // [ntiles] steps of this launch done
+    ChainCtl* ctl;
+    int ntiles;
+};
+
+constexpr int kChainDeps = 32;
+
 // Velocity output of the moments pass (whole-fluid velocity, Eq. 12 text).
 struct MomOut {
     double* ux;
@@ -144,6 +164,11 @@ struct Step {
                                  int parity, uint32_t* err, cudaStream_t s);
     // resident CTAs per SM of that kernel (0 if not available)
     static cudaError_t ring_ctas_per_sm(int D, int* out);
+    // chained steps (lbm_chain.cuh, FP64): nsteps steps in one launch of `grid`
+    // CTAs over tiles of the bidirectional march of W = 64 threads per group
+    static cudaError_t chain(const RunDesc* d_runs, const ChainTiles& ct, int nsteps, int parity, int rot, int grid,
+                             uint32_t* err, cudaStream_t s);
+    static cudaError_t chain_ctas_per_sm(int* out);
     // resident CTAs per SM of the bidirectional march with strips of W threads
     static cudaError_t bidir_ctas_per_sm(int W, int* out);
 };

@@ -5,6 +5,7 @@
 
 #include <atomic>
 
+#include "lbm_chain.cuh"
 #include "lbm_kernels.cuh"
 #include "lbm_ring.cuh"
 
@@ -282,6 +283,25 @@ cudaError_t Step<S, G>::bidir_ctas_per_sm(int W, int* out) {
 }
 
 template <typename S, bool G>
+cudaError_t Step<S, G>::chain(const RunDesc* d_runs, const ChainTiles& ct, int nsteps, int parity, int rot, int grid,
+                              uint32_t* err, cudaStream_t s) {
+    if constexpr (sizeof(S) != 8) {
+        return cudaErrorInvalidValue;   // FP64 only (lbm_chain.cuh)
+    } else {
+        if (ct.ntiles <= 0 || nsteps <= 0 || grid <= 0) return cudaSuccess;
+        k_chain_bidir<S, 64, G><<<grid, 128, 0, s>>>(d_runs, ct, nsteps, parity, rot, err);
+        return cudaGetLastError();
+    }
+}
+
+template <typename S, bool G>
+cudaError_t Step<S, G>::chain_ctas_per_sm(int* out) {
+    *out = 0;
+    if constexpr (sizeof(S) != 8) return cudaErrorInvalidValue;
+    else return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_chain_bidir<S, 64, G>, 128, 0);
+}
+
+template <typename S, bool G>
 cudaError_t Step<S, G>::step_ring(int D, const RunDesc* d_runs, const Tile* d_tiles, int ntiles, int* queue,
                                   int grid, int parity, uint32_t* err, cudaStream_t s) {
     if (grid <= 0 || ntiles <= 0) return cudaSuccess;
@@ -298,6 +318,7 @@ cudaError_t Step<S, G>::moments(int W, const RunDesc* d_runs, const Tile* d_tile
                                MomOut out, cudaStream_t s) {
     if (ntiles <= 0) return cudaSuccess;
     switch (W) {
+        case 32: k_step<S, 32, 1, false, G><<<ntiles, 32, 0, s>>>(d_runs, d_tiles, parity, out); break;
         case 64: k_step<S, 64, 1, false, G><<<ntiles, 64, 0, s>>>(d_runs, d_tiles, parity, out); break;
         case 128: k_step<S, 128, 1, false, G><<<ntiles, 128, 0, s>>>(d_runs, d_tiles, parity, out); break;
         case 256: k_step<S, 256, 1, false, G><<<ntiles, 256, 0, s>>>(d_runs, d_tiles, parity, out); break;

@@ -1,0 +1,86 @@
+"""Chained steps (many steps in one launch).  Every schedule gives the same bits, so each case compares populations
+(both buffers show in the velocity) with the staged march or the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+CHAIN = 12
+
+
+def Lattice(*a, **k):
+    from paper_0807_0602_gb300.build import build
+    build()
+    from paper_0807_0602_gb300 import lbm
+    return lbm.Lattice(*a, **k)
+
+
+def _run(nx, ny, kind, ratio=False, seed=5):
+    if kind == "box":
+        geom = W.periodic_box(nx, ny)
+    elif kind == "mask":
+        geom = W.periodic_box(nx, ny)
+        m = np.zeros((ny, nx), np.uint8)
+        m[0, : nx // 2] = 1
+        m[ny // 2, nx // 3: nx // 2] = 1
+        m[:, 0] |= np.arange(ny) % 5 == 0
+        geom["mask"] = m
+    else:
+        geom = W.capillary_geometry(nx, ny, nx // 8, nx - nx // 8, 0, ny - 3)
+    nA, nB = W.random_fields(geom, seed, 0.2, 1.2)
+    prm = W.params(0.9, 1.0, 0.9, -0.1, 0.05)
+    if ratio:
+        prm.update(alpha=(4 / 9, 0.8), mass=(1.0, 25 / 9))
+    return dict(geom=geom, params=prm, init=("fields", nA, nB))
+
+
+# one column of tiles and less, tile edges in both directions, one row, masks
+GRIDS = [(5, 4, "box"), (3, 1, "box"), (62, 8, "cap"), (63, 9, "cap"), (124, 7, "box"), (125, 33, "mask"),
+         (300, 40, "cap")]
+
+
+@pytest.mark.parametrize("nx,ny,kind", GRIDS)
+@pytest.mark.parametrize("rows", [1, 2, 5, 16])
+@pytest.mark.parametrize("ratio", [False, True])
+def test_chained_steps_equal_the_oracle(nx, ny, kind, rows, ratio):
+    run = _run(nx, ny, kind, ratio)
+    ref = oracle.OracleLattice(run["geom"], run["params"], run["init"][1], run["init"][2])
+    ref.step(41)
+    with Lattice(run, precision="f64", tile=(64, rows), kernel=(CHAIN, 4)) as lat:
+        lat.step(1)      # one step, an even and an odd number of chained ones
+        lat.step(30)
+        lat.step(7)
+        lat.step(3)
+        assert lat.status() == 0
+        assert np.array_equal(lat.populations(), ref.populations())
+        v, w = lat.velocity(), ref.velocity()
+        assert np.array_equal(v[0], w[0]) and np.array_equal(v[1], w[1])
+
+
+@pytest.mark.parametrize("chunk", [0, -1, 3])
+def test_chained_batch_with_log_equals_single_steps(chunk):
+    """Runs of uneven size share the chain; the log cuts it at its records."""
+    runs = [_run(90, 14, "cap", seed=1), _run(200, 33, "cap", seed=2), _run(64, 50, "cap", seed=3)]
+    kw = dict(precision="f64", log_every=10, log_capacity=16, graph_chunk=chunk)
+    with Lattice(runs, tile=(64, 3), kernel=(CHAIN, 4), **kw) as a, Lattice(runs, tile=(128, 4), kernel=(6, 4), **kw) as b:
+        for n in (4, 31, 25):
+            a.step(n)
+            b.step(n)
+        for r in range(3):
+            assert np.array_equal(a.populations(r), b.populations(r))
+            assert np.array_equal(a.log(r), b.log(r))
+
+
+def test_chain_is_refused_outside_fp64_and_its_tilings():
+    from paper_0807_0602_gb300 import _lib as L
+    with Lattice(_run(64, 18, "cap"), precision="f32") as lat:
+        with pytest.raises(L.LbmError):
+            lat.schedule = (64, 4, CHAIN, 4)
+    with Lattice(_run(64, 18, "cap"), precision="f64") as lat:
+        before = lat.schedule
+        for bad in ((128, 4, CHAIN, 4), (64, 4, CHAIN, 3), (64, 0, CHAIN, 4)):
+            with pytest.raises(L.LbmError):
+                lat.schedule = bad
+        assert lat.schedule == before
