@@ -137,11 +137,11 @@ typedef void (*lbm_free_fn)(void* ctx, void* ptr, size_t bytes, void* stream);
  *               where NVRTC is available; left out otherwise).  These are
  *               real steps: tilings change only the schedule, and results
  *               are bit-identical for every tiling.
- * tile_w        CTA width (64, 128 or 256 threads; 0 = default 128);
- * tile_h        rows marched per CTA (0 = default 4, clamped to ny).
- *               The step kernel starts as LBM_KERNEL_SMEM where it takes the
- *               tiling (else LBM_KERNEL_REGISTER); autotune or
- *               lbm_set_schedule change it.
+ * tile_w        a hint (64, 128 or 256; 0 = default 128), and
+ * tile_h        another (0 = default 4): the library chooses the step kernel
+ *               and its tiling from the precision and the runs' sizes, and
+ *               lbm_get_schedule reports them; autotune, lbm_set_tiling or
+ *               lbm_set_schedule change them.  Results do not depend on it.
  * graph_chunk   steps captured per CUDA graph when the log is off (0 = 64;
  *               -1 = launch every step directly).
  * rho_ref       FP16S shift per species (ignored otherwise).
@@ -203,7 +203,7 @@ typedef struct lbm_run_info {
     void* base[2];
 } lbm_run_info;
 
-/* Fills opt with the defaults documented above (FP32, no log, tile 128x4,
+/* Fills opt with the defaults documented above (FP32, no log, hint 128x4,
  * alpha 4/9, molecular mass 1). */
 void lbm_default_options(lbm_options* opt);
 
@@ -307,8 +307,8 @@ int lbm_set_columns(lbm_t* h, int run, int x0, int ncols, const void* buf, int o
 int lbm_get_tiling(const lbm_t* h, int* tile_w, int* tile_h);
 
 /* Selects a tiling (tile_w in {64,128,256}, tile_h >= 1) for the current step
- * kernel, or with the register kernel (LBM_KERNEL_REGISTER) if the current
- * kernel does not take that tiling.  Results do not depend on it. */
+ * kernel, or with a march (LBM_KERNEL_SMEM, else LBM_KERNEL_REGISTER) if the
+ * current kernel does not take that tiling.  Results do not depend on it. */
 int lbm_set_tiling(lbm_t* h, int tile_w, int tile_h);
 
 /* Full schedule of the step kernel: tiling (tile_w, tile_h) plus the kernel
@@ -326,7 +326,7 @@ int lbm_set_tiling(lbm_t* h, int tile_w, int tile_h);
  *                         <= 128, FP64 <= 64);
  *   LBM_KERNEL_SPLIT      one thread per species and node;
  *   LBM_KERNEL_PREFETCH   through registers, rows prefetched into L2;
- *   LBM_KERNEL_SMEM       parked in shared memory (the default; FP64 tile_w <= 128);
+ *   LBM_KERNEL_SMEM       parked in shared memory (FP64 tile_w <= 128);
  *   LBM_KERNEL_PAIR       two columns per thread (tile_w <= 128, FP64 64; nx >= 4);
  *   LBM_KERNEL_TILE       one node per thread over tile_w x (tile_h + 2)
  *                         threads (tile_w in {32, 64}, tile_h in {6, 14, 30},

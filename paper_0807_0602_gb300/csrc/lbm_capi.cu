@@ -651,6 +651,51 @@ struct Sched {
     int W, R, kvar, depth;
 };
 
+// The schedule of a handle that nobody has chosen one for, by the size of its
+// runs.  Measured on a GB300, us per step:
+//   - FP32 and FP16S up to 600 000 nodes: one node per thread (32 x 6 tiles).
+//     Every load of a tile is in flight at once, and small grids are bound by
+//     that latency: 256 x 32 2.4 (bidirectional 3.3, staged march 128 x 4 8.0),
+//     1024 x 66 4.0 (4.6, 8.2), 4095 x 67 with two masses 8.6 (10.3, 11.8),
+//     16 droplets of 256 x 128 19.4 (21.1, 23.3); 8192 x 160 43 (37.4, 43).
+//   - larger ones: the bidirectional march, tiles of 12 rows or fewer so that
+//     they fill whole waves of resident CTAs: 8192 x 160 37.4, FP16S 31.9
+//     (staged march 43.0, 35.0), 256 droplets 288 (308), 64 uneven capillaries
+//     499 (531).
+//   - FP64 from 30 000 nodes on: chained steps, tiles low enough for about 1000
+//     of them: 2048 x 130 154 (staged march 209), nine 128 x 80 droplets 88
+//     (164); below that (256 x 32: 22, 83) the bidirectional march with tiles
+//     of two rows.
+Sched default_schedule(lbm_t* h) {
+    double nodes = 0.0, strip_rows = 0.0;
+    int maxny = 1, minnx = 1 << 30;
+    for (const RunDesc& rd : h->runs) {
+        nodes += rd.nodes;
+        strip_rows += (double)((rd.nx + 61) / 62) * rd.ny;
+        maxny = std::max(maxny, rd.ny);
+        minnx = std::min(minnx, rd.nx);
+    }
+    if (h->precision == LBM_F64) {
+        if (nodes < 30000) return {64, std::min(2, maxny), 9, 4};
+        return {64, std::max(1, std::min({(int)(strip_rows / 900.0), 16, maxny})), 12, 4};
+    }
+    if (nodes <= 600000 && minnx >= 4) return {32, 6, 8, 4};
+    int R = std::min(12, maxny), per_sm = 0, dev = 0, sms = 0;
+    if (dispatch_step(h, [&](auto L) { return L.bidir_ctas_per_sm(64, &per_sm); }) == cudaSuccess && per_sm > 0 &&
+        cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0) {
+        const long long slots = (long long)per_sm * sms;
+        const long long waves = (bidir_tiles(h, 64, R) + slots - 1) / slots;
+        if (waves <= 8) {   // beyond that the last wave is a small share
+            const int Rw = wave_height(h, 64, (int)waves);
+            if (Rw > 0) R = std::min(R, Rw);
+        }
+    } else {
+        cudaGetLastError();
+    }
+    return {64, R, 9, 4};
+}
+
 // Times candidate tilings on the live state: the steps taken are real steps
 // (every tiling computes the same bits), only their schedule differs.
 int autotune(lbm_t* h, int64_t* n) {
@@ -957,13 +1002,10 @@ int create_impl(int n, const lbm_geometry* g, const double* G_AB, const double* 
     if (e != cudaSuccess) return fail(cuda_fail(h, e));
     // the host vectors above were read by async copies from pageable memory
     if (cudaStreamSynchronize(h->stream) != cudaSuccess) return fail(LBM_ECUDA);
-    const int W = opt.tile_w ? opt.tile_w : 128;
-    const int R = opt.tile_h ? opt.tile_h : 4;
-    // default kernel: the shared-memory-staged march, or the register march
-    // for tilings it does not take
-    h->kvar = schedule_ok(h, W, R, 6, 4) ? 6 : 0;
-    h->depth = 4;
-    if ((rc = upload_tiles(h, W, R))) return fail(rc);
+    const Sched sd = default_schedule(h);
+    h->kvar = sd.kvar;
+    h->depth = sd.depth;
+    if ((rc = upload_tiles(h, sd.W, sd.R))) return fail(rc);
     if (opt.log_every > 0) {
         e = issue_log(h, 0, h->stream);
         if (e != cudaSuccess) return fail(cuda_fail(h, e));
@@ -1213,9 +1255,10 @@ int lbm_get_tiling(const lbm_t* h, int* tile_w, int* tile_h) {
 int lbm_set_tiling(lbm_t* h, int tile_w, int tile_h) {
     if (!h) return LBM_EINVAL;
     if (!schedule_ok(h, tile_w, tile_h, h->kvar, h->depth)) {
-        // the current kernel does not take this tiling: the register march does
-        if (!schedule_ok(h, tile_w, tile_h, 0, 4)) return LBM_EINVAL;
-        h->kvar = 0;
+        // the current kernel does not take this tiling: a march does
+        const int march = schedule_ok(h, tile_w, tile_h, 6, 4) ? 6 : 0;
+        if (!schedule_ok(h, tile_w, tile_h, march, 4)) return LBM_EINVAL;
+        h->kvar = march;
         h->depth = 4;
     }
     h->tuned = true;
@@ -1288,8 +1331,8 @@ int lbm_save(lbm_t* h, const char* path) {
     hd.nruns = h->nruns;
     hd.log_every = h->opt.log_every;
     hd.log_capacity = h->opt.log_capacity;
-    hd.tile_w = h->tile_w;
-    hd.tile_h = h->tile_h;
+    hd.tile_w = h->opt.tile_w;   // the options' values: schedules are chosen anew on load
+    hd.tile_h = h->opt.tile_h;
     hd.t = h->t;
     hd.nlog = h->nlog;
     hd.rho_ref[0] = h->opt.rho_ref[0];

@@ -1,4 +1,6 @@
-"""Chained steps (many steps in one launch).  Every schedule gives the same bits, so each case compares populations
+"""Chained steps (many steps in one launch), the overlapping launches of the
+node-tile and bidirectional kernels, and the schedules that handles start
+with.  Every schedule gives the same bits, so each case compares populations
 (both buffers show in the velocity) with the staged march or the oracle."""
 import numpy as np
 import pytest
@@ -84,3 +86,41 @@ def test_chain_is_refused_outside_fp64_and_its_tilings():
             with pytest.raises(L.LbmError):
                 lat.schedule = bad
         assert lat.schedule == before
+
+
+# grids on both sides of the sizes at which the starting schedule changes
+@pytest.mark.parametrize("prec,nx,ny", [("f32", 33, 7), ("f32", 3, 5), ("f32", 300, 40), ("f32", 4000, 149),
+                                        ("f32", 4001, 150), ("f32", 1300, 700), ("f16s", 300, 40),
+                                        ("f16s", 4001, 150), ("f64", 100, 40), ("f64", 300, 99), ("f64", 300, 101)])
+def test_starting_schedule_gives_the_same_bits(prec, nx, ny):
+    run = _run(nx, ny, "cap" if nx > 8 else "box")
+    kw = dict(precision=prec, rho_ref=(1.0, 1.0))
+    with Lattice(run, **kw) as a, Lattice(run, tile=(128, 4), kernel=(6, 4), **kw) as b:
+        for n in (1, 18, 5):
+            a.step(n)
+            b.step(n)
+        assert np.array_equal(a.populations().view(np.uint8), b.populations().view(np.uint8))
+        va, vb = a.velocity(), b.velocity()
+        assert np.array_equal(va[0], vb[0]) and np.array_equal(va[1], vb[1])
+
+
+def test_pair_kernel_tiles_give_the_whole_velocity():
+    run = _run(300, 40, "cap")
+    with Lattice(run, precision="f32") as a, Lattice(run, precision="f32", tile=(64, 8), kernel=(7, 4)) as b:
+        a.step(6)
+        b.step(6)
+        for p, q in zip(a.velocity(), b.velocity()):
+            assert np.array_equal(p, q)
+
+
+def test_checkpoint_of_a_starting_schedule_loads(tmp_path):
+    run = _run(300, 40, "cap")
+    from paper_0807_0602_gb300.lbm import Lattice as Lat
+    for prec in ("f32", "f64"):
+        with Lattice(run, precision=prec) as a:
+            a.step(9)
+            a.save(str(tmp_path / prec))
+            a.step(8)
+            with Lat.load(str(tmp_path / prec)) as b:
+                b.step(8)
+                assert np.array_equal(a.populations(), b.populations())
