@@ -71,6 +71,13 @@ int mlp_gradients(mlp_t* h, const float* x, const float* t, int n, float* grad, 
  * batch before the update. */
 int mlp_train_step(mlp_t* h, const float* x, const float* t, int n, float lr, float* loss);
 
+/* `steps` training steps as above on minibatches of n rows gathered from
+ * x[rows][6] and t[rows][3]: step s trains on the rows idx[s n .. s n + n)
+ * (device int64; a number outside [0, rows) reads row 0).  loss (nullable)
+ * receives the `steps` losses. */
+int mlp_train_steps(mlp_t* h, const float* x, const float* t, int64_t rows, const int64_t* idx, int n, int steps,
+                    float lr, float* loss);
+
 /* Number of Adam steps taken since creation or the last mlp_set_params. */
 int64_t mlp_step_count(const mlp_t* h);
 

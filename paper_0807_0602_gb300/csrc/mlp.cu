@@ -229,10 +229,12 @@ __global__ void __launch_bounds__(kThreads) k_fwd(Dev d, const float* __restrict
 
 // Forward and backward pass of 16 MT rows: layer inputs and dL/dz of every
 // layer in bfloat16 (the operands of the weight gradients), dL/dz in FP32
-// (the bias gradients) and the squared error per 16 rows.
+// (the bias gradients) and the squared error per 16 rows.  idx: the batch is
+// the rows idx[0 .. n) of X and T (nullptr: the first n rows); gathering them
+// here costs a load in front of the chain instead of two kernels per batch.
 template <int MT>
 __global__ void __launch_bounds__(kThreads) k_train(Dev d, const float* __restrict__ X, const float* __restrict__ T,
-                                                    int n) {
+                                                    const long long* __restrict__ idx, long long nrows, int n) {
     __shared__ __align__(16) __nv_bfloat16 act[2][16 * MT][kLd];
     __shared__ float sq[MT][48];   // squared errors of each 16 rows, row by row
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, q = lane & 3;
@@ -245,9 +247,14 @@ __global__ void __launch_bounds__(kThreads) k_train(Dev d, const float* __restri
     // element e of mma tile mt of this lane: row row0 + row(mt, e / 2)
     auto row = [&](int mt, int e) { return 16 * mt + g + 8 * e; };
     auto live = [&](int mt, int e) { return row0 + row(mt, e) < n; };
+    auto source = [&](int r) -> long long {   // row of X and T (row 0 for a number out of range)
+        if (!idx) return r;
+        const long long i = idx[r];
+        return i >= 0 && i < nrows ? i : 0;
+    };
     float xv = 0.0f;
     const int xr = tid >> 4, xc = tid & 15;
-    if (xr < 16 * MT && row0 + xr < n && xc < 6) xv = X[(long long)(row0 + xr) * 6 + xc];
+    if (xr < 16 * MT && row0 + xr < n && xc < 6) xv = X[source(row0 + xr) * 6 + xc];
     const uint2 w0 = reinterpret_cast<const uint2*>(d.wf[0])[warp * 32 + lane];
     Frag128 w[2], w3;
     w[0].load(d.wf[1], warp, lane);
@@ -258,7 +265,7 @@ __global__ void __launch_bounds__(kThreads) k_train(Dev d, const float* __restri
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const int cc = 2 * q + (e & 1);
-            if (cc < 3 && live(warp, e >> 1)) t3[e] = T[(long long)(row0 + row(warp, e >> 1)) * 3 + cc];
+            if (cc < 3 && live(warp, e >> 1)) t3[e] = T[source(row0 + row(warp, e >> 1)) * 3 + cc];
             if (cc < 3) b3[e & 1] = d.theta[BOFF(3) + cc];
         }
     }
@@ -623,20 +630,35 @@ int forward_impl(mlp_t* h, const float* x, int n, float* y) {
 }
 
 // Forward, backward and the chunk partials of every gradient.
-int grad_impl(mlp_t* h, const float* x, const float* t, int n, int* chunks) {
+int grad_impl(mlp_t* h, const float* x, const float* t, int n, int* chunks, const long long* idx = nullptr,
+              long long nrows = 0) {
     const int tiles = (n + 15) / 16, n16 = tiles * 16;
     *chunks = (n16 + kChunkRows - 1) / kChunkRows;
     // 16 rows per CTA while every tile has an SM of its own, then 32 (4096 rows: the
     // whole gradient 18.7 us against 24.5 with 16, measured with split sums)
     cudaError_t e = tiles <= h->sms
-                        ? launch_pdl(k_train<1>, dim3(tiles), kThreads, h->stream, h->d, x, t, n)
-                        : launch_pdl(k_train<2>, dim3((tiles + 1) / 2), kThreads, h->stream, h->d, x, t, n);
+                        ? launch_pdl(k_train<1>, dim3(tiles), kThreads, h->stream, h->d, x, t, idx, nrows, n)
+                        : launch_pdl(k_train<2>, dim3((tiles + 1) / 2), kThreads, h->stream, h->d, x, t, idx, nrows, n);
     if (e == cudaSuccess)
         e = launch_pdl(k_wgrad, dim3(kWgradBlocks, *chunks), kWgradThreads, h->stream, h->d, n16);
     return e == cudaSuccess ? MLP_OK : fail(e);
 }
 
 constexpr int kUpdateGrid = (MLP_N_PARAMS + 127) / 128;
+
+// One training step on the first n rows, or on the rows idx[0 .. n).
+int train_impl(mlp_t* h, const float* x, const float* t, int n, float lr, float* loss, const long long* idx = nullptr,
+               long long nrows = 0) {
+    int chunks = 0;
+    const int rc = grad_impl(h, x, t, n, &chunks, idx, nrows);
+    if (rc) return rc;
+    h->steps += 1;
+    const double c1 = 1.0 / (1.0 - std::pow(0.9, (double)h->steps));
+    const double c2 = 1.0 / (1.0 - std::pow(0.999, (double)h->steps));
+    const cudaError_t e = launch_pdl(k_update<true>, dim3(kUpdateGrid), 128, h->stream, h->d, chunks, n,
+                                     (float*)nullptr, loss, lr, (float)c1, (float)c2);
+    return e == cudaSuccess ? MLP_OK : fail(e);
+}
 
 }  // namespace
 
@@ -735,15 +757,19 @@ int mlp_gradients(mlp_t* h, const float* x, const float* t, int n, float* grad, 
 
 int mlp_train_step(mlp_t* h, const float* x, const float* t, int n, float lr, float* loss) {
     if (!h || !x || !t || n < 1 || n > h->max_batch || !std::isfinite(lr)) return MLP_EINVAL;
-    int chunks = 0;
-    int rc = grad_impl(h, x, t, n, &chunks);
-    if (rc) return rc;
-    h->steps += 1;
-    const double c1 = 1.0 / (1.0 - std::pow(0.9, (double)h->steps));
-    const double c2 = 1.0 / (1.0 - std::pow(0.999, (double)h->steps));
-    cudaError_t e = launch_pdl(k_update<true>, dim3(kUpdateGrid), 128, h->stream, h->d, chunks, n, (float*)nullptr,
-                               loss, lr, (float)c1, (float)c2);
-    return e == cudaSuccess ? MLP_OK : fail(e);
+    return train_impl(h, x, t, n, lr, loss);
+}
+
+int mlp_train_steps(mlp_t* h, const float* x, const float* t, int64_t rows, const int64_t* idx, int n, int steps,
+                    float lr, float* loss) {
+    if (!h || !x || !t || !idx || rows < 1 || n < 1 || n > h->max_batch || steps < 0 || !std::isfinite(lr))
+        return MLP_EINVAL;
+    for (int s = 0; s < steps; ++s) {
+        const int rc = train_impl(h, x, t, n, lr, loss ? loss + s : nullptr,
+                                  reinterpret_cast<const long long*>(idx) + (size_t)s * n, rows);
+        if (rc) return rc;
+    }
+    return MLP_OK;
 }
 
 int64_t mlp_step_count(const mlp_t* h) { return h ? h->steps : -1; }

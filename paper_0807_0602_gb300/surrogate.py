@@ -32,6 +32,8 @@ MLP_SIGNATURES = {
                                      ctypes.c_void_p, ctypes.c_void_p]),
     "mlp_train_step": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int,
                                       ctypes.c_float, ctypes.c_void_p]),
+    "mlp_train_steps": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64,
+                                       ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_float, ctypes.c_void_p]),
     "mlp_step_count": (ctypes.c_int64, [ctypes.c_void_p]),
     "mlp_destroy": (None, [ctypes.c_void_p]),
 }
@@ -136,6 +138,18 @@ class Network:
                                         x.shape[0], float(lr), ctypes.c_void_p(loss.data_ptr())), "mlp_train_step")
         return loss
 
+    def train_steps(self, x, t, idx, lr: float):
+        """One training step per row of ``idx`` ([steps, n] row numbers of x
+        and t, the minibatches); returns the losses [steps]."""
+        x, t = self._dev(x, N_IN), self._dev(t, N_OUT)
+        idx = self._torch.as_tensor(idx).to(device="cuda", dtype=self._torch.int64).contiguous()
+        assert idx.dim() == 2 and x.shape[0] == t.shape[0]
+        loss = self._torch.empty(idx.shape[0], dtype=self._torch.float32, device="cuda")
+        _check(self._lib.mlp_train_steps(self._h, ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(t.data_ptr()),
+                                         x.shape[0], ctypes.c_void_p(idx.data_ptr()), idx.shape[1], idx.shape[0],
+                                         float(lr), ctypes.c_void_p(loss.data_ptr())), "mlp_train_steps")
+        return loss
+
 
 class Normalizer:
     """Per-column affine map to zero mean, unit spread (host-side data handling)."""
@@ -168,9 +182,11 @@ class Surrogate:
         Td = torch.as_tensor(self.tn.fwd(T), dtype=torch.float32, device="cuda")
         n = Xd.shape[0]
         losses = []
-        for s in range(steps):
-            idx = torch.as_tensor(rng.choice(n, size=min(batch, n), replace=False), device="cuda")
-            losses.append(self.net.train_step(Xd[idx], Td[idx], lr))
+        # blocks of steps: the next block's minibatches are drawn while the GPU
+        # trains on this one's
+        for s in range(0, steps, 64):
+            idx = np.stack([rng.choice(n, size=min(batch, n), replace=False) for _ in range(min(64, steps - s))])
+            losses.append(self.net.train_steps(Xd, Td, idx, lr))
         return torch.cat(losses).cpu().numpy()
 
     def predict(self, X) -> np.ndarray:

@@ -51,3 +51,20 @@ def test_forward_and_gradients_at_tile_edges(case):
             off += size
             assert np.max(np.abs(gk - bk)) <= 2e-2 * np.max(np.abs(bk)), (n, a, b, size)
     net.close()
+
+
+@pytest.mark.parametrize("n", [1, 16, 65, 512])
+def test_gathered_minibatches_equal_single_steps(n):
+    """train_steps on row numbers = train_step on the gathered rows, bit for bit
+    (rows repeat and are out of order; n = 512 fills one chunk of the sums)."""
+    import torch
+    from paper_0807_0602_gb300 import surrogate
+    rows = 700
+    a, th, X, T = _net(rows)
+    b = surrogate.Network(max_batch=rows, params=th.astype(np.float32))
+    idx = np.random.default_rng(3).integers(0, rows, size=(5, n))
+    la = a.train_steps(X, T, idx, 1e-3).cpu().numpy()
+    lb = torch.cat([b.train_step(X[i], T[i], 1e-3) for i in idx]).cpu().numpy()
+    assert np.array_equal(la, lb) and np.array_equal(a.params, b.params) and a.steps == b.steps == 5
+    a.close()
+    b.close()
