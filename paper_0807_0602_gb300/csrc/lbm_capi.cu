@@ -520,19 +520,12 @@ bool schedule_ok(const lbm_t* h, int W, int R, int kvar, int depth) {
     return true;
 }
 
-// Issues the log sequence for the state in buffer `parity`.
+// Issues one log record of the state in buffer `parity`.
 cudaError_t issue_log(lbm_t* h, int parity, cudaStream_t s) {
-    sc::LogCtl lc = logctl(h);
-    cudaError_t e = dispatch(h->precision, [&](auto L) {
-        return L.track(h->d_runs, h->nruns, h->track_cap, parity, h->d_first, lc, nullptr, s);
+    return dispatch(h->precision, [&](auto L) {
+        return L.log(h->d_runs, h->nruns, h->d_rows, (int)h->rows.size(), h->track_cap, parity, h->d_partials,
+                     h->d_first, logctl(h), h->d_err, s);
     });
-    if (e != cudaSuccess) return e;
-    e = dispatch(h->precision, [&](auto L) {
-        return L.mass(h->d_runs, h->nruns, h->d_rows, (int)h->rows.size(), parity, h->d_partials, nullptr, lc, 1,
-                      h->d_err, s);
-    });
-    if (e != cudaSuccess) return e;
-    return sc::launch_log_advance(lc, s);
 }
 
 int get_graph(lbm_t* h, int parity, int steps, int with_log, cudaGraphExec_t* out) {
@@ -976,7 +969,7 @@ int create_impl(int n, const lbm_geometry* g, const double* G_AB, const double* 
             return fail(LBM_ECUDA);
         for (int r = 0; r < n; ++r) h->runs[r].log = h->d_log + (size_t)r * opt.log_capacity * 6;
     }
-    h->d_logcount = static_cast<long long*>(dalloc(h, sizeof(long long)));
+    h->d_logcount = static_cast<long long*>(dalloc(h, 2 * sizeof(long long)));
     h->d_err = static_cast<uint32_t*>(dalloc(h, sizeof(uint32_t)));
     h->d_partials = static_cast<double*>(dalloc(h, (size_t)2 * sc::kMassChunks * h->rows.size() * sizeof(double)));
     h->d_mass = static_cast<double*>(dalloc(h, (size_t)2 * n * sizeof(double)));
@@ -991,7 +984,8 @@ int create_impl(int n, const lbm_geometry* g, const double* G_AB, const double* 
     if (!h->d_logcount || !h->d_err || !h->d_partials || !h->d_mass || !h->d_zout || !h->d_first || !h->d_rows ||
         !h->d_runs)
         return fail(LBM_ENOMEM);
-    if (cudaMemsetAsync(h->d_logcount, 0, sizeof(long long), h->stream) != cudaSuccess ||
+    if (cudaMemsetAsync(h->d_logcount, 0, 2 * sizeof(long long), h->stream) != cudaSuccess ||
+        cudaMemsetAsync(h->d_first, 0x7f, (size_t)4 * n * sizeof(int), h->stream) != cudaSuccess ||   // kNoFront
         cudaMemsetAsync(h->d_err, 0, sizeof(uint32_t), h->stream) != cudaSuccess ||
         cudaMemcpyAsync(h->d_rows, h->rows.data(), h->rows.size() * sizeof(int2), cudaMemcpyHostToDevice,
                         h->stream) != cudaSuccess ||
@@ -1032,7 +1026,7 @@ int fetch_fields(lbm_t* h, int run, double* a, double* b, int on_device, bool ve
     cudaError_t e;
     if (!velocity) {
         e = dispatch(h->precision,
-                     [&](auto L) { return L.densities(h->d_runs, run, (int)(h->t & 1), rd.nodes, da, db, h->stream); });
+                     [&](auto L) { return L.densities(h->d_runs, run, (int)(h->t & 1), rd.nx, rd.ny, da, db, h->stream); });
     } else if (h->t == 0) {
         e = cudaMemsetAsync(da, 0, nn * sizeof(double), h->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(db, 0, nn * sizeof(double), h->stream);
@@ -1134,9 +1128,8 @@ int lbm_interface_positions(lbm_t* h, int run, double* z_bulk, double z_prec[2])
     if (check_run(h, run) || !z_bulk || !z_prec) return LBM_EINVAL;
     const RunDesc& rd = h->runs[run];
     if (rd.y_bot < 0 || rd.y_top < 0 || rd.y_top - rd.y_bot < 2 || rd.cap_x1 <= rd.cap_x0) return LBM_ESTATE;
-    sc::LogCtl lc{nullptr, 1, 0};
     cudaError_t e = dispatch(h->precision, [&](auto L) {
-        return L.track(h->d_runs, h->nruns, h->track_cap, (int)(h->t & 1), h->d_first, lc, h->d_zout, h->stream);
+        return L.track(h->d_runs, h->nruns, h->track_cap, (int)(h->t & 1), h->d_first, h->d_zout, h->stream);
     });
     if (e != cudaSuccess) return cuda_fail(h, e);
     double z[3];
@@ -1171,10 +1164,9 @@ int lbm_get_log(lbm_t* h, int run, double* rec, int capacity, int* n_rec) {
 
 int lbm_mass(lbm_t* h, int run, double M[2]) {
     if (check_run(h, run) || !M) return LBM_EINVAL;
-    sc::LogCtl lc{nullptr, 1, 0};
     cudaError_t e = dispatch(h->precision, [&](auto L) {
         return L.mass(h->d_runs, h->nruns, h->d_rows, (int)h->rows.size(), (int)(h->t & 1), h->d_partials, h->d_mass,
-                      lc, 0, h->d_err, h->stream);
+                      h->d_err, h->stream);
     });
     if (e != cudaSuccess) return cuda_fail(h, e);
     CK(h, cudaMemcpyAsync(M, h->d_mass + 2 * run, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));

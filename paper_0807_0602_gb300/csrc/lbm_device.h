@@ -81,6 +81,9 @@ inline void fill_coef_f32(RunDesc& rd) {
 // column chunks (CTAs) per row of the mass reduction
 constexpr int kMassChunks = 4;
 
+// "no failing column" of the front scan (a byte pattern, so that a memset sets it)
+constexpr int kNoFront = 0x7f7f7f7f;
+
 // collided columns per strip of the persistent ring kernel (LBM_KERNEL_RING)
 constexpr int kRingWc = 120;
 
@@ -123,7 +126,7 @@ struct MomOut {
 
 // Shared state of the logging kernels.
 struct LogCtl {
-    long long* count;   // records written so far (device)
+    long long* count;   // records written so far (device); count[1]: CTAs done with the next one
     int cap;            // ring capacity
     int log_every;
 };
@@ -177,13 +180,16 @@ struct Step {
 template <typename S>
 struct Launch {
     static cudaError_t init(const RunDesc* d_runs, int nruns, int max_nodes, cudaStream_t s);
-    static cudaError_t densities(const RunDesc* d_runs, int run, int parity, int nodes, double* nA,
+    static cudaError_t densities(const RunDesc* d_runs, int run, int parity, int nx, int ny, double* nA,
                                  double* nB, cudaStream_t s);
-    static cudaError_t track(const RunDesc* d_runs, int nruns, int max_cap, int parity, int* first, LogCtl lc,
-                             double* zout, cudaStream_t s);
+    // fronts to zout[nruns][3]; first[4 nruns]: kNoFront before and after
+    static cudaError_t track(const RunDesc* d_runs, int nruns, int max_cap, int parity, int* first, double* zout,
+                             cudaStream_t s);
     static cudaError_t mass(const RunDesc* d_runs, int nruns, const int2* d_rows, int nrows, int parity,
-                            double* d_partials, double* d_mass, LogCtl lc, int write_log, uint32_t* d_err,
-                            cudaStream_t s);
+                            double* d_partials, double* d_mass, uint32_t* d_err, cudaStream_t s);
+    // one log record of every run (fronts and masses)
+    static cudaError_t log(const RunDesc* d_runs, int nruns, const int2* d_rows, int nrows, int max_cap, int parity,
+                           double* d_partials, int* first, LogCtl lc, uint32_t* d_err, cudaStream_t s);
     static cudaError_t export_pops(const RunDesc* d_runs, int run, int parity, int nx, int ny, void* out,
                                    cudaStream_t s);
     static cudaError_t import_pops(const RunDesc* d_runs, int run, int parity, int nx, int ny, const void* in,
@@ -194,8 +200,6 @@ struct Launch {
     static cudaError_t set_cols(const RunDesc* d_runs, int run, int parity, int ny, int x0, int ncols,
                                 const void* in, cudaStream_t s);
 };
-
-cudaError_t launch_log_advance(LogCtl lc, cudaStream_t s);
 
 extern template struct Launch<double>;
 extern template struct Launch<float>;

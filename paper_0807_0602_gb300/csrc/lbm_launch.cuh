@@ -328,37 +328,51 @@ cudaError_t Step<S, G>::moments(int W, const RunDesc* d_runs, const Tile* d_tile
 }
 
 template <typename S>
-cudaError_t Launch<S>::densities(const RunDesc* d_runs, int run, int parity, int nodes, double* nA, double* nB,
+cudaError_t Launch<S>::densities(const RunDesc* d_runs, int run, int parity, int nx, int ny, double* nA, double* nB,
                                  cudaStream_t s) {
-    k_densities<S><<<clamp_grid((nodes + 255) / 256, 4096), 256, 0, s>>>(d_runs, run, parity, nA, nB);
+    const int threads = nx <= 128 ? 128 : 256;
+    k_densities<S><<<dim3((nx + threads - 1) / threads, ny < 65535 ? ny : 65535), threads, 0, s>>>(d_runs, run, parity,
+                                                                                                 nA, nB);
     return cudaGetLastError();
 }
 
+// CTAs of a front scan over the longest capillary
+static inline int track_chunks(int max_cap) { return (max_cap + kTrackCols - 1) / kTrackCols; }
+
 template <typename S>
-cudaError_t Launch<S>::track(const RunDesc* d_runs, int nruns, int max_cap, int parity, int* first, LogCtl lc,
-                             double* zout, cudaStream_t s) {
+cudaError_t Launch<S>::track(const RunDesc* d_runs, int nruns, int max_cap, int parity, int* first, double* zout,
+                             cudaStream_t s) {
     if (nruns <= 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(first, 0x7f, (size_t)4 * nruns * sizeof(int), s);   // kNoFront
-    if (e != cudaSuccess) return e;
     if (max_cap > 0) {
-        k_track_scan<S><<<dim3((max_cap + kTrackThreads - 1) / kTrackThreads, nruns), kTrackThreads, 0, s>>>(
-            d_runs, parity, first);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        k_track_scan<S><<<dim3(track_chunks(max_cap), nruns), kTrackThreads, 0, s>>>(d_runs, parity, first);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
     }
-    k_track_final<S><<<nruns, 32, 0, s>>>(d_runs, parity, first, lc, zout);
-    return cudaGetLastError();
+    return launch_step(k_track_final<S>, nruns, 32, s, d_runs, parity, first, zout);
 }
 
 template <typename S>
 cudaError_t Launch<S>::mass(const RunDesc* d_runs, int nruns, const int2* d_rows, int nrows, int parity,
-                            double* d_partials, double* d_mass, LogCtl lc, int write_log, uint32_t* d_err,
-                            cudaStream_t s) {
+                            double* d_partials, double* d_mass, uint32_t* d_err, cudaStream_t s) {
     if (nruns <= 0) return cudaSuccess;
     k_mass_rows<S><<<dim3(nrows, kMassChunks), kMassThreads, 0, s>>>(d_runs, d_rows, parity, d_partials);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_mass_final<<<nruns, kMassThreads, 0, s>>>(d_runs, d_partials, d_mass, lc, write_log, d_err);
+    k_mass_final<<<nruns, kMassThreads, 0, s>>>(d_runs, d_partials, d_mass, d_err);
     return cudaGetLastError();
+}
+
+template <typename S>
+cudaError_t Launch<S>::log(const RunDesc* d_runs, int nruns, const int2* d_rows, int nrows, int max_cap, int parity,
+                           double* d_partials, int* first, LogCtl lc, uint32_t* d_err, cudaStream_t s) {
+    if (nruns <= 0) return cudaSuccess;
+    const int chunks = max_cap > 0 ? track_chunks(max_cap) : 0;
+    const long long grid = (long long)nrows * kMassChunks + (long long)chunks * nruns;
+    if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
+    cudaError_t e = launch_step(k_log_rows<S>, (int)grid, kMassThreads, s, d_runs, d_rows, nrows, chunks, parity,
+                                d_partials, first);
+    if (e != cudaSuccess) return e;
+    return launch_step(k_log_final<S>, nruns, kMassThreads, s, d_runs, parity, d_partials, first, lc, d_err);
 }
 
 template <typename S>
@@ -378,21 +392,36 @@ cudaError_t Launch<S>::import_pops(const RunDesc* d_runs, int run, int parity, i
     return cudaGetLastError();
 }
 
+// Thread block of a column copy: as many threads along a row as it has
+// accesses (at most 256), the rest of 256 threads along the rows.
+static inline dim3 cols_block(int accesses) {
+    int tx = 1;
+    while (tx < accesses && tx < 256) tx *= 2;
+    return dim3(tx, 256 / tx);
+}
+
 template <typename S>
 cudaError_t Launch<S>::get_cols(const RunDesc* d_runs, int run, int parity, int ny, int x0, int ncols, void* out,
                                 cudaStream_t s) {
-    const long long total = 18LL * ny * ncols;
-    k_get_cols<S><<<clamp_grid((total + 255) / 256, 4096), 256, 0, s>>>(d_runs, run, parity, x0, ncols,
-                                                                        static_cast<S*>(out));
+    // 16-byte accesses where every row of the window and of the buffer starts
+    // on one (rows of the populations start LBM_COL0 elements into a row of a
+    // multiple of 64)
+    constexpr int V = 16 / (int)sizeof(S);
+    S* o = static_cast<S*>(out);
+    const bool wide = x0 % V == 0 && ncols % V == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+    const dim3 block = cols_block(wide ? ncols / V : ncols);
+    const int grid = clamp_grid((18LL * ny + block.y - 1) / block.y, 8192);
+    if (wide) k_get_cols<S, V><<<grid, block, 0, s>>>(d_runs, run, parity, x0, ncols, o);
+    else k_get_cols<S, 1><<<grid, block, 0, s>>>(d_runs, run, parity, x0, ncols, o);
     return cudaGetLastError();
 }
 
 template <typename S>
 cudaError_t Launch<S>::set_cols(const RunDesc* d_runs, int run, int parity, int ny, int x0, int ncols,
                                 const void* in, cudaStream_t s) {
-    const long long total = 18LL * ny * ncols;
-    k_set_cols<S><<<clamp_grid((total + 255) / 256, 4096), 256, 0, s>>>(d_runs, run, parity, x0, ncols,
-                                                                        static_cast<const S*>(in));
+    const dim3 block = cols_block(ncols);
+    k_set_cols<S><<<clamp_grid((18LL * ny + block.y - 1) / block.y, 8192), block, 0, s>>>(
+        d_runs, run, parity, x0, ncols, static_cast<const S*>(in));
     return cudaGetLastError();
 }
 
