@@ -303,6 +303,15 @@ int lbm_populations(lbm_t* h, int run, void* out, int on_device);
 int lbm_get_columns(lbm_t* h, int run, int x0, int ncols, void* buf, int on_device);
 int lbm_set_columns(lbm_t* h, int run, int x0, int ncols, const void* buf, int on_device);
 
+/* `steps` steps of one capillary held as n x-slabs (lattices of one run with
+ * two halo columns on each side, as above) in ring order: after every step of
+ * all of them, each slab's halo columns are overwritten with the neighbours'
+ * edge columns, the same copies as lbm_get_columns / lbm_set_columns in one
+ * launch.  The slabs are distinct handles of one precision, stream and device
+ * with equal ny and nx >= 8, 1 <= n <= 32 (LBM_EINVAL otherwise, nothing
+ * stepped).  Asynchronous; returns the first error of a step. */
+int lbm_step_slabs(lbm_t* const* slabs, int n, int64_t steps);
+
 /* Tiling in use (CTA width, rows per CTA). */
 int lbm_get_tiling(const lbm_t* h, int* tile_w, int* tile_h);
 

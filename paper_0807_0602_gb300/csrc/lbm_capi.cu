@@ -1237,6 +1237,37 @@ int lbm_set_columns(lbm_t* h, int run, int x0, int ncols, const void* buf, int o
     return columns_io(h, run, x0, ncols, const_cast<void*>(buf), on_device, true);
 }
 
+int lbm_step_slabs(lbm_t* const* slabs, int n, int64_t steps) {
+    if (!slabs || n < 1 || n > sc::kMaxSlabs || steps < 0) return LBM_EINVAL;
+    for (int p = 0; p < n; ++p) {
+        const lbm_t* h = slabs[p];
+        if (!h || h->nruns != 1 || h->runs[0].nx < 8 || h->precision != slabs[0]->precision ||
+            h->runs[0].ny != slabs[0]->runs[0].ny || h->stream != slabs[0]->stream)
+            return LBM_EINVAL;
+        for (int q = 0; q < p; ++q)
+            if (slabs[q] == h) return LBM_EINVAL;
+        cudaPointerAttributes a, a0;
+        CK(slabs[0], cudaPointerGetAttributes(&a, h->d_runs));
+        CK(slabs[0], cudaPointerGetAttributes(&a0, slabs[0]->d_runs));
+        if (a.device != a0.device) return LBM_EINVAL;
+    }
+    for (int64_t j = 0; j < steps; ++j) {
+        sc::SlabHalos sh{};
+        sh.n = n;
+        for (int p = 0; p < n; ++p) {
+            const int rc = lbm_step(slabs[p], 1);
+            if (rc) return rc;
+            sh.run[p] = slabs[p]->d_runs;
+            sh.parity[p] = (int)(slabs[p]->t & 1);
+        }
+        const cudaError_t e = dispatch(slabs[0]->precision, [&](auto L) {
+            return L.slab_halos(sh, slabs[0]->runs[0].ny, slabs[0]->stream);
+        });
+        if (e != cudaSuccess) return cuda_fail(slabs[0], e);
+    }
+    return LBM_OK;
+}
+
 int lbm_get_tiling(const lbm_t* h, int* tile_w, int* tile_h) {
     if (!h || !tile_w || !tile_h) return LBM_EINVAL;
     *tile_w = h->tile_w;

@@ -124,6 +124,14 @@ struct MomOut {
     int nx;
 };
 
+// x-slabs of one process in ring order (k_slab_halos).
+constexpr int kMaxSlabs = 32;
+struct SlabHalos {
+    const RunDesc* run[kMaxSlabs];
+    int parity[kMaxSlabs];   // buffer of the slab's current populations
+    int n;
+};
+
 // Shared state of the logging kernels.
 struct LogCtl {
     long long* count;   // records written so far (device); count[1]: CTAs done with the next one
@@ -197,6 +205,7 @@ struct Launch {
     // column window [x0, x0 + ncols) to / from a packed [18][ny][ncols] buffer
     static cudaError_t get_cols(const RunDesc* d_runs, int run, int parity, int ny, int x0, int ncols, void* out,
                                 cudaStream_t s);
+    static cudaError_t slab_halos(const SlabHalos& h, int ny, cudaStream_t s);
     static cudaError_t set_cols(const RunDesc* d_runs, int run, int parity, int ny, int x0, int ncols,
                                 const void* in, cudaStream_t s);
 };

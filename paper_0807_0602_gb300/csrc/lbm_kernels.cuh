@@ -2282,6 +2282,23 @@ __global__ void k_set_cols(const RunDesc* __restrict__ runs, int run, int parity
     }
 }
 
+// Halo exchange among the x-slabs of one process, all copies in one launch:
+// blockIdx.y = 2 slab + side; the two halo columns of a side come from the
+// neighbour's edge columns (owned columns, which no copy writes).
+template <typename S>
+__global__ void k_slab_halos(SlabHalos h) {
+    step_ready();
+    const int side = blockIdx.y & 1, p = blockIdx.y >> 1;
+    const int q = (p + (side ? 1 : h.n - 1)) % h.n;
+    const RunDesc &to = *h.run[p], &from = *h.run[q];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, row = i >> 1, c = i & 1;
+    if (row >= 18 * to.ny) return;
+    const int ki = row / to.ny, y = row - ki * to.ny;
+    const int xf = (side ? 2 : from.nx - 4) + c, xt = (side ? to.nx - 2 : 0) + c;
+    const S v = static_cast<const S*>(from.buf[h.parity[q]])[ki * from.plane + (long long)y * from.pitch + xf];
+    set_with_images(static_cast<S*>(to.buf[h.parity[p]]) + ki * to.plane + (long long)y * to.pitch, xt, to.nx, v);
+}
+
 // ---- fronts (Numerical Results section, Figs. 6-8) -------------------------
 // Four tracked rows per run, scanned from cap_x0:
 //   g = 0, 1: the centre row(s) with v = phi = (n_A - n_B)/(n_A + n_B);

@@ -417,6 +417,20 @@ cudaError_t Launch<S>::get_cols(const RunDesc* d_runs, int run, int parity, int 
 }
 
 template <typename S>
+cudaError_t Launch<S>::slab_halos(const SlabHalos& h, int ny, cudaStream_t s) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((36 * ny + 127) / 128, 2 * h.n);
+    cfg.blockDim = dim3(128);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};   // as launch_step
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_slab_halos<S>, h);
+}
+
+template <typename S>
 cudaError_t Launch<S>::set_cols(const RunDesc* d_runs, int run, int parity, int ny, int x0, int ncols,
                                 const void* in, cudaStream_t s) {
     const dim3 block = cols_block(ncols);

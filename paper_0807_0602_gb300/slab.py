@@ -20,6 +20,8 @@ send/recv (NCCL between GPUs, gloo between CPU processes).
 """
 from __future__ import annotations
 
+import ctypes
+
 import numpy as np
 
 HALO = 2   # columns of halo on each side
@@ -104,8 +106,28 @@ def exchange_local(slabs) -> None:
         s.set_halos(edges[(p - 1) % P][1], edges[(p + 1) % P][0])
 
 
+def _step_native(slabs, n: int) -> bool:
+    """The steps and exchanges of GPU slabs of one stream and device by one
+    library call (one copy kernel per step); False if these slabs need the
+    general exchange."""
+    from . import lbm as B
+    if not 1 <= len(slabs) <= 32 or any(type(s) is not Slab or type(s.lat) is not B.Lattice for s in slabs):
+        return False
+    lats = [s.lat for s in slabs]
+    one = lats[0]
+    if len({id(a) for a in lats}) != len(lats) or any(
+            not a._h or a.nruns != 1 or a.precision != one.precision or a.device != one.device
+            or a.stream.cuda_stream != one.stream.cuda_stream or a.shapes[0][0] != one.shapes[0][0] for a in lats):
+        return False
+    handles = (ctypes.c_void_p * len(lats))(*[a._h.value for a in lats])
+    B.L.check(one._lib.lbm_step_slabs(handles, len(lats), int(n)), "lbm_step")
+    return True
+
+
 def step_local(slabs, n: int) -> None:
     """n steps of the decomposed run held by one process."""
+    if n > 0 and _step_native(slabs, n):
+        return
     for _ in range(n):
         for s in slabs:
             s.step()
