@@ -646,15 +646,16 @@ struct Sched {
 
 // The schedule of a handle that nobody has chosen one for, by the size of its
 // runs.  Measured on a GB300, us per step:
-//   - FP32 and FP16S up to 600 000 nodes: one node per thread (32 x 6 tiles).
+//   - FP32 and FP16S up to 250 000 nodes: one node per thread (32 x 6 tiles).
 //     Every load of a tile is in flight at once, and small grids are bound by
 //     that latency: 256 x 32 2.4 (bidirectional 3.3, staged march 128 x 4 8.0),
-//     1024 x 66 4.0 (4.6, 8.2), 4095 x 67 with two masses 8.6 (10.3, 11.8),
-//     16 droplets of 256 x 128 19.4 (21.1, 23.3); 8192 x 160 43 (37.4, 43).
+//     1024 x 66 4.0 (4.6, 8.2); equal at 274 000 nodes (4095 x 67 with two
+//     masses 8.6, 8.7, 11.8), then behind: 16 droplets of 256 x 128 19.4
+//     (16.2, 23.3), 8192 x 160 43 (36.8, 43).
 //   - larger ones: the bidirectional march, tiles of 12 rows or fewer so that
-//     they fill whole waves of resident CTAs: 8192 x 160 37.4, FP16S 31.9
-//     (staged march 43.0, 35.0), 256 droplets 288 (308), 64 uneven capillaries
-//     499 (531).
+//     they fill whole waves of resident CTAs: 8192 x 160 36.8, FP16S 31.7
+//     (staged march 43.0, 35.0), 256 droplets 274 (308), 64 uneven capillaries
+//     488 (531).
 //   - FP64 from 30 000 nodes on: chained steps, tiles low enough for about 1000
 //     of them: 2048 x 130 154 (staged march 209), nine 128 x 80 droplets 88
 //     (164); below that (256 x 32: 22, 83) the bidirectional march with tiles
@@ -670,9 +671,11 @@ Sched default_schedule(lbm_t* h) {
     }
     if (h->precision == LBM_F64) {
         if (nodes < 30000) return {64, std::min(2, maxny), 9, 4};
-        return {64, std::max(1, std::min({(int)(strip_rows / 900.0), 16, maxny})), 12, 4};
+        // even heights: both groups of a tile march the same number of rows
+        const int R = std::max(1, std::min({(int)(strip_rows / 900.0), 16, maxny}));
+        return {64, R > 1 ? R & ~1 : R, 12, 4};
     }
-    if (nodes <= 600000 && minnx >= 4) return {32, 6, 8, 4};
+    if (nodes <= 250000 && minnx >= 4) return {32, 6, 8, 4};
     int R = std::min(12, maxny), per_sm = 0, dev = 0, sms = 0;
     if (dispatch_step(h, [&](auto L) { return L.bidir_ctas_per_sm(64, &per_sm); }) == cudaSuccess && per_sm > 0 &&
         cudaGetDevice(&dev) == cudaSuccess &&

@@ -1167,7 +1167,8 @@ __device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, con
     char* const udst = reinterpret_cast<char*>(dst - LBM_COL0);
     const unsigned xo = (unsigned)((sc.dcol ? tl.x0 - 1 + t : tl.x0) + LBM_COL0) * (unsigned)sizeof(S);
     const unsigned pitchB = (unsigned)pitch * (unsigned)sizeof(S), planeB = plane * (unsigned)sizeof(S);
-    const bool ghost = ghost_r(sc.xc, nx) | ghost_l(sc.xc, nx);
+    // bytes from the column to its periodic image (one at most with nx >= 4), 0 = none
+    const int image = (ghost_r(sc.xc, nx) + ghost_l(sc.xc, nx)) * (int)sizeof(S);
     auto pull_plain = [&](int k, int r) {
         // 64-bit row pointers plus multiples of the plane: one wide multiply-add
         // per access, an immediate offset where the plane is a constant
@@ -1236,10 +1237,14 @@ __device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, con
                 C fn[2][9];
                 relax<S>(cx, fc, ns, fn);
                 char* o = udst + (size_t)((unsigned)r * pitchB + xo);
+                for (int to = image;; to = 0) {   // once more for a column with a periodic image (rare)
 #pragma unroll
-                for (int q = 0; q < 18; ++q)
-                    enc(reinterpret_cast<S*>(o + (unsigned long long)planeB * (unsigned)q), fn[q / 9][q % 9],
-                        cx.sh.v[q / 9][grp(q % 9)]);
+                    for (int q = 0; q < 18; ++q)
+                        enc(reinterpret_cast<S*>(o + (unsigned long long)planeB * (unsigned)q), fn[q / 9][q % 9],
+                            cx.sh.v[q / 9][grp(q % 9)]);
+                    if (to == 0) break;
+                    o += to;
+                }
                 sm_prev = sm_cur;
                 continue;
             }
