@@ -38,6 +38,7 @@ struct RunDesc {
     // and both m_k are 1 (the step kernels of the standard model run then)
     double dA[2][3];
     int gen;
+    int ints;                 // FP64: equilibrium brackets on the integer pipe
     CoefF32 c32;
     double rho_ref[2];        // FP16S shift per species
     double thr;               // precursor threshold rho_bulk / 3

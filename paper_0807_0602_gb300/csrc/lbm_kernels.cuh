@@ -37,6 +37,9 @@
 #pragma once
 
 #include "lbm_device.h"
+#ifndef __CUDACC_RTC__   // (run-time compiled kernels keep the FP64 instructions: the same bits)
+#include "lbm_exact.h"
+#endif
 
 namespace sc {
 
@@ -241,6 +244,7 @@ struct StepCtx {
     C dA[2][3];   // A_g(alpha_k) - w_g (GEN only; 0 for a species with alpha_k = 4/9)
     bool body;    // a body force acts (gx or gy is not zero)
     bool unit[2]; // tau_k = 1
+    bool ints;    // equilibrium brackets on integers (FP64, RunDesc::ints)
     Shift<S> sh;
     // With m_k = 1 (not GEN), taum = tau and the weights of U are itau.
     __device__ __forceinline__ const C (&wU() const)[2] {
@@ -279,6 +283,7 @@ struct StepCtx {
             gy = (C)rd.gy;
             // by their bits: FP64 comparisons run on the FP64 pipe
             body = ((__double_as_longlong(rd.gx) | __double_as_longlong(rd.gy)) << 1) != 0;
+            ints = rd.ints != 0;
             unit[0] = __double_as_longlong(rd.itauA) == 0x3ff0000000000000LL;
             unit[1] = __double_as_longlong(rd.itauB) == 0x3ff0000000000000LL;
             if constexpr (GEN) {
@@ -425,29 +430,72 @@ __device__ __forceinline__ void div2(double a, double b, double d, double& qa, d
 // FP64 instruction counts: 329 per node before
 // these forms and div2, 254 with them (tau = 1; tile 64x8 of the bidirectional
 // march), 887 and 722 us per step of the 8192x160 grid.
+// With |u| < 0.2, almost everywhere, the brackets are formed on integers
+// (lbm_exact.h), and a relaxation with tau = 1 near equilibrium needs no
+// operation: 254 -> 151 FP64 instructions per node, 722 -> 490 us per step.
 template <typename C, bool GEN>
-__device__ __forceinline__ void feq_relax(C ux, C uy, C xx, C yy, C b, C wn0, C wn1, C wn5, const C (&dn)[3], C itau,
-                                          bool unit, const C (&f)[9], C (&fnew)[9]) {
+__device__ __forceinline__ void feq_relax(C ux, C uy, C xx, C yy, C usq, C wn0, C wn1, C wn5, const C (&dn)[3], C itau,
+                                          bool unit, bool ints, const C (&f)[9], C (&fnew)[9]) {
     using A = Ar<C>;
     C feq[9];
-    feq[0] = A::mul(wn0, A::sub(C(1), b));
     const C d = A::add(ux, uy), e = A::sub(uy, ux);
     const C cp[4] = {ux, uy, d, e}, cc[4] = {xx, yy, A::mul(d, d), A::mul(e, e)};
     constexpr int ia[4] = {1, 2, 5, 6}, ib[4] = {3, 4, 7, 8};
+    bool done = false;
+#ifndef __CUDACC_RTC__
+    if constexpr (sizeof(C) == 8) {
+        if (ints && (unsigned)__double2hiint(usq) < (unsigned)exact::kMaxUsqHigh) {
+            auto ub = [](double v) { return (exact::u64)__double_as_longlong(v); };
+            auto db = [](exact::u64 v) { return __longlong_as_double((long long)v); };
+            const exact::Fix b = exact::b_of(ub(usq));
+            feq[0] = A::mul(wn0, db(exact::rest(b)));
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const C wn = q < 2 ? wn1 : wn5;
-        const C t = A::mul(C(3), cp[q]), s = A::mul(C(4.5), cc[q]);
-        feq[ia[q]] = A::mul(wn, A::sub(A::add(s, A::add(t, C(1))), b));
-        feq[ib[q]] = A::mul(wn, A::sub(A::add(s, A::sub(C(1), t)), b));
+            for (int q = 0; q < 4; ++q) {
+                const C wn = q < 2 ? wn1 : wn5;
+                exact::u64 p, m;
+                exact::pair(ub(cp[q]), ub(cc[q]), b, p, m);
+                feq[ia[q]] = A::mul(wn, db(p));
+                feq[ib[q]] = A::mul(wn, db(m));
+            }
+            done = true;
+        }
+    }
+#endif
+    if (!done) {
+        const C b = A::mul(C(1.5), usq);
+        feq[0] = A::mul(wn0, A::sub(C(1), b));
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const C wn = q < 2 ? wn1 : wn5;
+            const C t = A::mul(C(3), cp[q]), s = A::mul(C(4.5), cc[q]);
+            feq[ia[q]] = A::mul(wn, A::sub(A::add(s, A::add(t, C(1))), b));
+            feq[ib[q]] = A::mul(wn, A::sub(A::add(s, A::sub(C(1), t)), b));
+        }
     }
     if constexpr (GEN) {
 #pragma unroll
         for (int i = 0; i < 9; ++i) feq[i] = A::add(feq[i], dn[grp(i)]);
     }
     if (unit) {
+        // tau = 1: f - (f - feq).  Where f and feq agree within a factor of two
+        // their difference is exact (Sterbenz), and so f minus it is feq itself;
+        // the factor is read off the high words (feq finite: n below 2^1000).
+        bool near = false;
+#ifndef __CUDACC_RTC__
+        if constexpr (sizeof(C) == 8) {
+            near = ints && ((unsigned)__double2hiint(wn0) & 0x7fffffffu) < 0x7e700000u && done;
 #pragma unroll
-        for (int i = 0; i < 9; ++i) fnew[i] = A::sub(f[i], A::sub(f[i], feq[i]));
+            for (int i = 0; i < 9; ++i)
+                near = near && (unsigned)(__double2hiint(f[i]) - __double2hiint(feq[i]) + 0x0fffff) < 0x1fffffu;
+        }
+#endif
+        if (near) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) fnew[i] = feq[i];
+        } else {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) fnew[i] = A::sub(f[i], A::sub(f[i], feq[i]));
+        }
     } else {
 #pragma unroll
         for (int i = 0; i < 9; ++i) fnew[i] = A::fma(-A::sub(f[i], feq[i]), itau, f[i]);   // Eq. 2
@@ -499,7 +547,7 @@ __device__ __forceinline__ void relax(const StepCtx<S, GEN>& cx, const typename 
 #pragma unroll
                 for (int g = 0; g < 3; ++g) dn[g] = A::mul(cx.dA[k][g], nk);   // free alpha_k
             }
-            feq_relax<C, GEN>(ux, uy, xx, yy, b, wn0, wn1, wn5, dn, cx.itau[k], cx.unit[k], fc[k], fnew[k]);
+            feq_relax<C, GEN>(ux, uy, xx, yy, usq, wn0, wn1, wn5, dn, cx.itau[k], cx.unit[k], cx.ints, fc[k], fnew[k]);
         } else {
             // Eqs. 3-5 by opposite pairs: feq(+-c) = wn (1 + 4.5 c^2 - b) +- 3 wn c;
             // Eq. 2 as f (1 - 1/tau) + feq / tau
@@ -811,7 +859,7 @@ __device__ __forceinline__ void collide_species(const StepCtx<S, GEN>& cx, int k
 #pragma unroll
             for (int g = 0; g < 3; ++g) dn[g] = A::mul(cx.dA[k][g], n);
         }
-        feq_relax<C, GEN>(ux, uy, xx, yy, b, wn0, wn1, wn5, dn, cx.itau[k], cx.unit[k], f, fnew);
+        feq_relax<C, GEN>(ux, uy, xx, yy, usq, wn0, wn1, wn5, dn, cx.itau[k], cx.unit[k], cx.ints, f, fnew);
     } else {
         const C om = C(1) - cx.itau[k], it = cx.itau[k];
         const C base = C(1) - b;
@@ -1045,7 +1093,7 @@ __global__ void __launch_bounds__(W, (kSmemMinBlocks<S, W>)) k_step_smem(const R
 // barrier of step 2 CTA-wide too, so that no group reuses its step-0 slot (at
 // step 4) before the other group has read it.
 template <typename S, int W>
-constexpr int kBidirMinBlocks = sizeof(typename Prec<S>::C) == 8 ? 1 : 512 / W;   // 64 registers
+constexpr int kBidirMinBlocks = sizeof(typename Prec<S>::C) == 8 ? 3 : 512 / W;   // FP64: 168 registers, else 64
 
 // bar.sync on barrier 1 or 2 (immediate ids: the kernel reserves three barriers) for N threads
 template <int N>
@@ -1231,7 +1279,7 @@ __device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, con
 #pragma unroll
                 for (int i = 0; i < 9; ++i)
                     fc[kk][i] = (kF && i == 0) ? C(0) : ps[grp_d][(k - 1) & 1][pidx(kk, i)][pc];
-            if ((unsigned)(r - pl0) < (unsigned)pln && !ghost) {
+            if ((unsigned)(r - pl0) < (unsigned)pln) {
                 NodeState<S> ns;
                 node_state<S, W>(cx, fc, 0u, sd, s_m, s_row, s_p, t, ns);
                 C fn[2][9];

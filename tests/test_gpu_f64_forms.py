@@ -30,3 +30,25 @@ def test_f64_forms_bit_equal(scale, tau, body):
             lat.step(4)
         got = lat.populations()
     assert np.all(np.isfinite(want)) and np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("tau", [(1.0, 1.0), (1.0, 1.3)])
+@pytest.mark.parametrize("lo,hi", [(0.9, 1.1), (0.02, 2.0)])
+def test_integer_forms_bit_equal_on_larger_grids(tau, lo, hi):
+    """From 30 000 nodes on the brackets are formed on integers where u.u is
+    below its bound (everywhere in the mild field, not so in the rough one)."""
+    from paper_0807_0602_gb300.build import build
+    build()
+    from paper_0807_0602_gb300.lbm import Lattice
+    geom = W.capillary_geometry(251, 130, 30, 220, 0, 117)
+    nA, nB = W.random_fields(geom, 4, lo, hi)
+    prm = W.params(0.9, *tau, -0.1, 0.07)
+    ref = oracle.OracleLattice(geom, prm, nA, nB)
+    ref.step(8)
+    with Lattice(dict(geom=geom, params=prm, init=("fields", nA, nB)), precision="f64") as lat:
+        lat.step(3)
+        for sched in ((128, 4, 6, 4), (64, 8, 9, 4), (128, 5, 4, 4), (32, 6, 8, 4), (64, 6, 11, 4)):
+            lat.schedule = sched
+            lat.step(1)
+        got = lat.populations()
+    assert np.all(np.isfinite(got)) and np.array_equal(got, ref.populations())
