@@ -311,6 +311,7 @@ template <typename S>
 struct NodeState {
     using C = typename Prec<S>::C;
     C n[2], jx[2], jy[2], ax[2], ay[2];
+    C wn1[2], wn5[2];   // w_1 n, w_5 n of the node (filled where the products are shared)
 };
 
 // wall sum of Eq. 11 over the solid neighbours, i ascending
@@ -328,10 +329,14 @@ __device__ __forceinline__ void wall_terms(unsigned m, C& Wx, C& Wy) {
     if (SOL(m, -1, 1)) { Wx = A::add(Wx, Wc::w5); Wy = A::sub(Wy, Wc::w5); }  // i = 8
 }
 
-template <typename S, int W, bool G, bool FULL = false>
+// PW: the products w_1 n and w_5 n of every node are shared too, in
+// pw[slot][species][axis, diagonal][column]: the FP64 march forms them once
+// per node instead of once per neighbour (4 instead of 20 multiplications;
+// 8192x160: 490 -> 442 us).
+template <typename S, int W, bool G, bool FULL = false, bool PW = false>
 __device__ __forceinline__ void node_state(const StepCtx<S, G>& cx, const typename Prec<S>::C (&fc)[2][9], unsigned m,
                                            const typename Prec<S>::C (*sd)[2][W], int s_m, int s_0, int s_p, int t,
-                                           NodeState<S>& ns) {
+                                           NodeState<S>& ns, const typename Prec<S>::C (*pw)[2][2][W] = nullptr) {
     using C = typename Prec<S>::C;
     using Wc = Wt<C>;
     using A = Ar<C>;
@@ -347,18 +352,32 @@ __device__ __forceinline__ void node_state(const StepCtx<S, G>& cx, const typena
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const int kb = 1 - k;
-        const C n1 = sd[s_0][kb][t + 1], n2 = sd[s_p][kb][t], n3 = sd[s_0][kb][t - 1], n4 = sd[s_m][kb][t],
-                n5 = sd[s_p][kb][t + 1], n6 = sd[s_p][kb][t - 1], n7 = sd[s_m][kb][t - 1], n8 = sd[s_m][kb][t + 1];
-        C Sx = A::fma(-Wc::w1, n3, A::mul(Wc::w1, n1));
-        Sx = A::fma(Wc::w5, n5, Sx);
-        Sx = A::fma(-Wc::w5, n6, Sx);
-        Sx = A::fma(-Wc::w5, n7, Sx);
-        Sx = A::fma(Wc::w5, n8, Sx);
-        C Sy = A::fma(-Wc::w1, n4, A::mul(Wc::w1, n2));
-        Sy = A::fma(Wc::w5, n5, Sy);
-        Sy = A::fma(Wc::w5, n6, Sy);
-        Sy = A::fma(-Wc::w5, n7, Sy);
-        Sy = A::fma(-Wc::w5, n8, Sy);
+        C Sx, Sy;
+        if constexpr (PW) {
+            const C p5 = pw[s_p][kb][1][t + 1], p6 = pw[s_p][kb][1][t - 1], p7 = pw[s_m][kb][1][t - 1],
+                    p8 = pw[s_m][kb][1][t + 1];
+            Sx = A::sub(pw[s_0][kb][0][t + 1], pw[s_0][kb][0][t - 1]);
+            Sx = A::sub(A::sub(A::add(Sx, p5), p6), p7);
+            Sx = A::add(Sx, p8);
+            Sy = A::sub(pw[s_p][kb][0][t], pw[s_m][kb][0][t]);
+            Sy = A::add(A::add(Sy, p5), p6);
+            Sy = A::sub(A::sub(Sy, p7), p8);
+            ns.wn1[k] = pw[s_0][k][0][t];
+            ns.wn5[k] = pw[s_0][k][1][t];
+        } else {
+            const C n1 = sd[s_0][kb][t + 1], n2 = sd[s_p][kb][t], n3 = sd[s_0][kb][t - 1], n4 = sd[s_m][kb][t],
+                    n5 = sd[s_p][kb][t + 1], n6 = sd[s_p][kb][t - 1], n7 = sd[s_m][kb][t - 1], n8 = sd[s_m][kb][t + 1];
+            Sx = A::fma(-Wc::w1, n3, A::mul(Wc::w1, n1));
+            Sx = A::fma(Wc::w5, n5, Sx);
+            Sx = A::fma(-Wc::w5, n6, Sx);
+            Sx = A::fma(-Wc::w5, n7, Sx);
+            Sx = A::fma(Wc::w5, n8, Sx);
+            Sy = A::fma(-Wc::w1, n4, A::mul(Wc::w1, n2));
+            Sy = A::fma(Wc::w5, n5, Sy);
+            Sy = A::fma(Wc::w5, n6, Sy);
+            Sy = A::fma(-Wc::w5, n7, Sy);
+            Sy = A::fma(-Wc::w5, n8, Sy);
+        }
         ns.ax[k] = -A::mul(cx.G, Sx);
         ns.ay[k] = -A::mul(cx.G, Sy);
     }
@@ -433,6 +452,8 @@ __device__ __forceinline__ void div2(double a, double b, double d, double& qa, d
 // With |u| < 0.2, almost everywhere, the brackets are formed on integers
 // (lbm_exact.h), and a relaxation with tau = 1 near equilibrium needs no
 // operation: 254 -> 151 FP64 instructions per node, 722 -> 490 us per step.
+// (Rounding the products w n times the bracket on integers as well, 30
+// instructions each, gained nothing: the chain of one node gets longer.)
 template <typename C, bool GEN>
 __device__ __forceinline__ void feq_relax(C ux, C uy, C xx, C yy, C usq, C wn0, C wn1, C wn5, const C (&dn)[3], C itau,
                                           bool unit, bool ints, const C (&f)[9], C (&fnew)[9]) {
@@ -504,7 +525,7 @@ __device__ __forceinline__ void feq_relax(C ux, C uy, C xx, C yy, C usq, C wn0, 
 
 // Steps 4-7: common velocity, shifted equilibria and BGK relaxation.
 // GEN: the equilibria carry dA_i n_k and U weighs m_k / tau_k.
-template <typename S, bool GEN>
+template <typename S, bool GEN, bool PW = false>
 __device__ __forceinline__ void relax(const StepCtx<S, GEN>& cx, const typename Prec<S>::C (&fc)[2][9],
                                            const NodeState<S>& ns, typename Prec<S>::C (&fnew)[2][9]) {
     using C = typename Prec<S>::C;
@@ -540,7 +561,8 @@ __device__ __forceinline__ void relax(const StepCtx<S, GEN>& cx, const typename 
         const C usq = kCanonical<C> ? A::add(xx, yy) : A::fma(ux, ux, yy);
         const C b = A::mul(C(1.5), usq);
         const C nk = ns.n[k];
-        const C wn0 = A::mul(Wc::w0, nk), wn1 = A::mul(Wc::w1, nk), wn5 = A::mul(Wc::w5, nk);
+        const C wn0 = A::mul(Wc::w0, nk), wn1 = PW ? ns.wn1[k] : A::mul(Wc::w1, nk),
+                wn5 = PW ? ns.wn5[k] : A::mul(Wc::w5, nk);
         if constexpr (kCanonical<C>) {
             C dn[3];
             if constexpr (GEN) {
@@ -584,15 +606,16 @@ __device__ __forceinline__ void relax(const StepCtx<S, GEN>& cx, const typename 
 // periodic images at x = nx, nx + 1 and x = -2, -1 (ghost columns), so that
 // every source row a later step reads is one contiguous window; gr / gl give
 // the offsets of those images from the node (0 = none).
-template <typename S, int W, int MODE, bool GH, bool G>
+template <typename S, int W, int MODE, bool GH, bool G, bool PW>
 __device__ __forceinline__ void collide_node(const StepCtx<S, G>& cx, const typename Prec<S>::C (&fc)[2][9], unsigned m,
                                              const typename Prec<S>::C (*sd)[2][W], int s_m, int s_0, int s_p, int t,
                                              S* __restrict__ dst, unsigned plane, unsigned o, MomOut mo,
-                                             long long mo_idx, int gr = 0, int gl = 0) {
+                                             long long mo_idx, const typename Prec<S>::C (*pw)[2][2][W], int gr = 0,
+                                             int gl = 0) {
     using C = typename Prec<S>::C;
     using A = Ar<C>;
     NodeState<S> ns;
-    node_state<S, W, G, MODE == 1>(cx, fc, m, sd, s_m, s_0, s_p, t, ns);
+    node_state<S, W, G, MODE == 1, PW>(cx, fc, m, sd, s_m, s_0, s_p, t, ns, pw);
     if (MODE == 1) {
         C rho, px, py;
         if constexpr (G) {
@@ -611,7 +634,7 @@ __device__ __forceinline__ void collide_node(const StepCtx<S, G>& cx, const type
         return;
     }
     C fnew[2][9];
-    relax<S>(cx, fc, ns, fnew);
+    relax<S, G, PW>(cx, fc, ns, fnew);
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         S* d = dst + ((unsigned)(k * 9) * plane + o);
@@ -629,15 +652,16 @@ __device__ __forceinline__ void collide_node(const StepCtx<S, G>& cx, const type
 }
 
 // Dispatch: the ghost-writing variant only for the edge columns.
-template <typename S, int W, int MODE, bool G>
+template <typename S, int W, int MODE, bool G, bool PW = false>
 __device__ __forceinline__ void collide_any(const StepCtx<S, G>& cx, const typename Prec<S>::C (&fc)[2][9], unsigned m,
                                             const typename Prec<S>::C (*sd)[2][W], int s_m, int s_0, int s_p, int t,
                                             S* __restrict__ dst, unsigned plane, unsigned o, MomOut mo,
-                                            long long mo_idx, int gr, int gl) {
+                                            long long mo_idx, int gr, int gl,
+                                            const typename Prec<S>::C (*pw)[2][2][W] = nullptr) {
     if (gr | gl)
-        collide_node<S, W, MODE, true>(cx, fc, m, sd, s_m, s_0, s_p, t, dst, plane, o, mo, mo_idx, gr, gl);
+        collide_node<S, W, MODE, true, G, PW>(cx, fc, m, sd, s_m, s_0, s_p, t, dst, plane, o, mo, mo_idx, pw, gr, gl);
     else
-        collide_node<S, W, MODE, false>(cx, fc, m, sd, s_m, s_0, s_p, t, dst, plane, o, mo, mo_idx, 0, 0);
+        collide_node<S, W, MODE, false, G, PW>(cx, fc, m, sd, s_m, s_0, s_p, t, dst, plane, o, mo, mo_idx, pw, 0, 0);
 }
 
 // Column bookkeeping of a strip: thread t <-> column x0 - 1 + t (wrapped).
@@ -1095,6 +1119,10 @@ __global__ void __launch_bounds__(W, (kSmemMinBlocks<S, W>)) k_step_smem(const R
 template <typename S, int W>
 constexpr int kBidirMinBlocks = sizeof(typename Prec<S>::C) == 8 ? 3 : 512 / W;   // FP64: 168 registers, else 64
 
+// Dynamic shared memory of the march (FP64: 2 x 5 density slots of products)
+template <typename S, int W>
+constexpr int kBidirDynSmem = sizeof(typename Prec<S>::C) == 8 ? 10 * 2 * 2 * W * 8 : 0;
+
 // bar.sync on barrier 1 or 2 (immediate ids: the kernel reserves three barriers) for N threads
 template <int N>
 __device__ __forceinline__ void bar_group(int g) {
@@ -1121,6 +1149,16 @@ __device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, con
     constexpr int PW = kF ? W - 2 : W;  // staged columns
     __shared__ C sd[2 * NS][2][W];      // [group * NS + step slot][species][column]
     __shared__ C ps[2][2][NP][PW];      // [group][step parity][population][column]
+    // FP64: the products w n beside the densities (bidir_smem bytes of dynamic
+    // shared memory; run-time compiled kernels do without)
+#ifdef LBM_JIT_GRID
+    constexpr bool kPw = false;
+    C(*pw)[2][2][W] = nullptr;
+#else
+    constexpr bool kPw = !kF;
+    extern __shared__ __align__(16) unsigned char bidir_dyn[];
+    C(*pw)[2][2][W] = reinterpret_cast<C(*)[2][2][W]>(bidir_dyn);
+#endif
 
     const Tile tl = tiles[tile];
     const RunDesc& rd = runs[tl.run];
@@ -1161,6 +1199,17 @@ __device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, con
     auto pidx = [&](int kk, int i) { return kF ? kk * 8 + i - 1 : kk * 9 + i; };
     const int pc = kF ? t - 1 : t;
 
+    auto put_dens = [&](int sl, C nA, C nB) {
+        sd[sl][0][t] = nA;
+        sd[sl][1][t] = nB;
+        if constexpr (kPw) {
+            using Wc = Wt<C>;
+            pw[sl][0][0][t] = Ar<C>::mul(Wc::w1, nA);
+            pw[sl][0][1][t] = Ar<C>::mul(Wc::w5, nA);
+            pw[sl][1][0][t] = Ar<C>::mul(Wc::w1, nB);
+            pw[sl][1][1][t] = Ar<C>::mul(Wc::w5, nB);
+        }
+    };
     auto pull = [&](int k, unsigned& smask) {
         const int r = row_at(k);
         const RowIdx q = rows_of(r, ny);
@@ -1184,8 +1233,7 @@ __device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, con
                 }
             }
         }
-        sd[slot(grp_d, k)][0][t] = nA;
-        sd[slot(grp_d, k)][1][t] = nB;
+        put_dens(slot(grp_d, k), nA, nB);
     };
 
     // Plain rows: no solid among the 3x3 neighbours of any column of the strip
@@ -1238,8 +1286,7 @@ __device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, con
             f[kk][7] = dec(at(9 * kk + 7, op, 1), cx.sh.v[kk][2]);
             f[kk][8] = dec(at(9 * kk + 8, op, -1), cx.sh.v[kk][2]);
         }
-        sd[slot(grp_d, k)][0][t] = dens9(f[0]);
-        sd[slot(grp_d, k)][1][t] = dens9(f[1]);
+        put_dens(slot(grp_d, k), dens9(f[0]), dens9(f[1]));
         if (sc.coll && k < nrows) {
 #pragma unroll
             for (int kk = 0; kk < 2; ++kk)
@@ -1281,9 +1328,9 @@ __device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, con
                     fc[kk][i] = (kF && i == 0) ? C(0) : ps[grp_d][(k - 1) & 1][pidx(kk, i)][pc];
             if ((unsigned)(r - pl0) < (unsigned)pln) {
                 NodeState<S> ns;
-                node_state<S, W>(cx, fc, 0u, sd, s_m, s_row, s_p, t, ns);
+                node_state<S, W, G, false, kPw>(cx, fc, 0u, sd, s_m, s_row, s_p, t, ns, pw);
                 C fn[2][9];
-                relax<S>(cx, fc, ns, fn);
+                relax<S, G, kPw>(cx, fc, ns, fn);
                 char* o = udst + (size_t)((unsigned)r * pitchB + xo);
                 for (int to = image;; to = 0) {   // once more for a column with a periodic image (rare)
 #pragma unroll
@@ -1297,9 +1344,9 @@ __device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, con
                 continue;
             }
             const int rw = rows_of(r, ny).rw;
-            collide_any<S, W, 0>(cx, fc, sm_prev, sd, s_m, s_row, s_p, t, dst, plane,
+            collide_any<S, W, 0, G, kPw>(cx, fc, sm_prev, sd, s_m, s_row, s_p, t, dst, plane,
                                  (unsigned)(rw * pitch + sc.xc), MomOut{nullptr, nullptr, 0}, 0, ghost_r(sc.xc, nx),
-                                 ghost_l(sc.xc, nx));
+                                 ghost_l(sc.xc, nx), pw);
         }
         sm_prev = sm_cur;
     }

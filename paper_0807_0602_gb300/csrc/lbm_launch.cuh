@@ -28,8 +28,9 @@ static inline cudaError_t ensure_dynamic_smem(const void* fn, int bytes, std::at
 // Launches a step kernel so that its CTAs may start while the kernel before it
 // on the stream ends (it waits itself, step_ready).
 template <typename... P, typename... Q>
-static cudaError_t launch_step(void (*fn)(P...), int grid, int threads, cudaStream_t s, Q... args) {
+static cudaError_t launch_step_dyn(void (*fn)(P...), int grid, int threads, int smem, cudaStream_t s, Q... args) {
     cudaLaunchConfig_t cfg{};
+    cfg.dynamicSmemBytes = smem;
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(threads);
     cfg.stream = s;
@@ -39,6 +40,11 @@ static cudaError_t launch_step(void (*fn)(P...), int grid, int threads, cudaStre
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, fn, P(args)...);
+}
+
+template <typename... P, typename... Q>
+static cudaError_t launch_step(void (*fn)(P...), int grid, int threads, cudaStream_t s, Q... args) {
+    return launch_step_dyn(fn, grid, threads, 0, s, args...);
 }
 
 static inline int clamp_grid(long long want, int cap) {
@@ -219,12 +225,29 @@ cudaError_t Step<S, G>::step_tile(int W, int R, const RunDesc* d_runs, const Til
     }
 }
 
+// Raises the shared memory limit of the FP64 marches (47 KB static and the products).
+template <typename S, bool G>
+static cudaError_t bidir_smem() {
+    if constexpr (kBidirDynSmem<S, 64> == 0) {
+        return cudaSuccess;
+    } else {
+        static std::atomic<unsigned long long> step{0}, chain{0};
+        const cudaError_t e = ensure_dynamic_smem((const void*)k_step_bidir<S, 64, G>, kBidirDynSmem<S, 64>, step);
+        if (e != cudaSuccess) return e;
+        return ensure_dynamic_smem((const void*)k_chain_bidir<S, 64, G>, kBidirDynSmem<S, 64>, chain);
+    }
+}
+
 template <typename S, bool G>
 cudaError_t Step<S, G>::step_bidir(int W, const RunDesc* d_runs, const Tile* d_tiles, int ntiles, int parity,
                                   cudaStream_t s) {
     if (ntiles <= 0) return cudaSuccess;
     switch (W) {
-        case 64: return launch_step(k_step_bidir<S, 64, G>, ntiles, 128, s, d_runs, d_tiles, parity);
+        case 64: {
+            const cudaError_t e = bidir_smem<S, G>();
+            if (e != cudaSuccess) return e;
+            return launch_step_dyn(k_step_bidir<S, 64, G>, ntiles, 128, kBidirDynSmem<S, 64>, s, d_runs, d_tiles, parity);
+        }
         case 128:
             if constexpr (sizeof(typename Prec<S>::C) == 8) return cudaErrorInvalidValue;
             else return launch_step(k_step_bidir<S, 128, G>, ntiles, 256, s, d_runs, d_tiles, parity);
@@ -274,7 +297,11 @@ template <typename S, bool G>
 cudaError_t Step<S, G>::bidir_ctas_per_sm(int W, int* out) {
     *out = 0;
     switch (W) {
-        case 64: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_step_bidir<S, 64, G>, 128, 0);
+        case 64: {
+            const cudaError_t e = bidir_smem<S, G>();
+            if (e != cudaSuccess) return e;
+            return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_step_bidir<S, 64, G>, 128, kBidirDynSmem<S, 64>);
+        }
         case 128:
             if constexpr (sizeof(typename Prec<S>::C) == 8) return cudaErrorInvalidValue;
             else return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_step_bidir<S, 128, G>, 256, 0);
@@ -289,7 +316,9 @@ cudaError_t Step<S, G>::chain(const RunDesc* d_runs, const ChainTiles& ct, int n
         return cudaErrorInvalidValue;   // FP64 only (lbm_chain.cuh)
     } else {
         if (ct.ntiles <= 0 || nsteps <= 0 || grid <= 0) return cudaSuccess;
-        k_chain_bidir<S, 64, G><<<grid, 128, 0, s>>>(d_runs, ct, nsteps, parity, rot, err);
+        const cudaError_t e = bidir_smem<S, G>();
+        if (e != cudaSuccess) return e;
+        k_chain_bidir<S, 64, G><<<grid, 128, kBidirDynSmem<S, 64>, s>>>(d_runs, ct, nsteps, parity, rot, err);
         return cudaGetLastError();
     }
 }
@@ -297,8 +326,13 @@ cudaError_t Step<S, G>::chain(const RunDesc* d_runs, const ChainTiles& ct, int n
 template <typename S, bool G>
 cudaError_t Step<S, G>::chain_ctas_per_sm(int* out) {
     *out = 0;
-    if constexpr (sizeof(S) != 8) return cudaErrorInvalidValue;
-    else return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_chain_bidir<S, 64, G>, 128, 0);
+    if constexpr (sizeof(S) != 8) {
+        return cudaErrorInvalidValue;
+    } else {
+        const cudaError_t e = bidir_smem<S, G>();
+        if (e != cudaSuccess) return e;
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_chain_bidir<S, 64, G>, 128, kBidirDynSmem<S, 64>);
+    }
 }
 
 template <typename S, bool G>
