@@ -1258,14 +1258,15 @@ __device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, con
         }
     }
     // byte offset of this thread's column in row 0, from LBM_COL0 columns
-    // before column 0 (idle threads of a narrow last strip repeat column x0)
+    // before column 0
     const char* const usrc = reinterpret_cast<const char*>(src - LBM_COL0);
     char* const udst = reinterpret_cast<char*>(dst - LBM_COL0);
-    const unsigned xo = (unsigned)((sc.dcol ? tl.x0 - 1 + t : tl.x0) + LBM_COL0) * (unsigned)sizeof(S);
+    const unsigned xo = (unsigned)(tl.x0 - 1 + t + LBM_COL0) * (unsigned)sizeof(S);
     const unsigned pitchB = (unsigned)pitch * (unsigned)sizeof(S), planeB = plane * (unsigned)sizeof(S);
     // bytes from the column to its periodic image (one at most with nx >= 4), 0 = none
     const int image = (ghost_r(sc.xc, nx) + ghost_l(sc.xc, nx)) * (int)sizeof(S);
     auto pull_plain = [&](int k, int r) {
+        if (!sc.dcol) return;   // idle warps of a narrow last strip
         // 64-bit row pointers plus multiples of the plane: one wide multiply-add
         // per access, an immediate offset where the plane is a constant
         const char* o = usrc + (size_t)((unsigned)r * pitchB + xo);
