@@ -77,6 +77,7 @@ struct lbm_s {
     uint32_t* d_err = nullptr;
     double* d_scratch = nullptr;   // [2][max_nodes] FP64 for host copies
     void* d_popscratch = nullptr;  // [18][max_nodes] storage type
+    sc::Shape shape{};             // the runs' size if they are alike
     int max_nodes = 0;
     int64_t t = 0;
     long long nlog = 0;            // host mirror of the log count
@@ -428,7 +429,7 @@ cudaError_t issue_step(lbm_t* h, int parity, cudaStream_t s) {
     if (h->kvar == 7)
         return dispatch_step(h, [&](auto L) { return L.step_pair(W, h->d_runs, h->d_tiles, nt, parity, s); });
     if (h->kvar == 9)
-        return dispatch_step(h, [&](auto L) { return L.step_bidir(W, h->d_runs, h->d_tiles, nt, parity, s); });
+        return dispatch_step(h, [&](auto L) { return L.step_bidir(W, h->d_runs, h->d_tiles, nt, parity, h->shape, s); });
     if (h->kvar == 8)
         return dispatch_step(h,
                              [&](auto L) { return L.step_tile(W, h->tile_h, h->d_runs, h->d_tiles, nt, parity, s); });
@@ -983,8 +984,12 @@ int create_impl(int n, const lbm_geometry* g, const double* G_AB, const double* 
             h->track_cap = std::max(h->track_cap, rd.cap_x1 - rd.cap_x0);
     h->d_rows = static_cast<int2*>(dalloc(h, h->rows.size() * sizeof(int2)));
     h->d_runs = static_cast<RunDesc*>(dalloc(h, (size_t)n * sizeof(RunDesc)));
+    h->shape = {h->runs[0].nx, h->runs[0].ny, h->runs[0].pitch, (unsigned)h->runs[0].plane};
     double nodes = 0.0;
-    for (const RunDesc& rd : h->runs) nodes += rd.nodes;
+    for (const RunDesc& rd : h->runs) {
+        nodes += rd.nodes;
+        if (rd.nx != h->shape.nx || rd.ny != h->shape.ny) h->shape.nx = 0;
+    }
     for (RunDesc& rd : h->runs) {
         rd.err = h->d_err;
         // below that a step is bound by one node's chain of operations, which

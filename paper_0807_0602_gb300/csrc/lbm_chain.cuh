@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(2 * W, (kBidirMinBlocks<S, W>)) k_chain_bidir(
                                                                                ChainTiles ct, int nsteps, int parity,
                                                                                int rot, uint32_t* err) {
     chain_run<2 * W>(ct, nsteps, parity, rot, err, [&](int tile, int par, auto ready) {
-        bidir_tile<S, W, G, false>(runs, ct.tiles, tile, par, ready);
+        bidir_tile<S, W, G, false, false>(runs, ct.tiles, tile, par, Shape{}, ready);
     });
 }
 

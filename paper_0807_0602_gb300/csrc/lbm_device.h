@@ -118,6 +118,13 @@ struct ChainTiles {
 
 constexpr int kChainDeps = 32;
 
+// Size of every run of a handle whose runs are alike (nx = 0: they are not).
+// As kernel parameters these are known to be the same for all threads.
+struct Shape {
+    int nx, ny, pitch;
+    unsigned plane;
+};
+
 // Velocity output of the moments pass (whole-fluid velocity, Eq. 12 text).
 struct MomOut {
     double* ux;
@@ -166,7 +173,7 @@ struct Step {
     static cudaError_t step_tile(int W, int R, const RunDesc* d_runs, const Tile* d_tiles, int ntiles, int parity,
                                  cudaStream_t s);
     static cudaError_t step_bidir(int W, const RunDesc* d_runs, const Tile* d_tiles, int ntiles, int parity,
-                                  cudaStream_t s);
+                                  const Shape& shape, cudaStream_t s);
     static cudaError_t moments(int W, const RunDesc* d_runs, const Tile* d_tiles, int ntiles, int parity,
                                MomOut out, cudaStream_t s);
     // persistent ring kernel (FP32 / FP16S storage, D row slots): `grid` CTAs

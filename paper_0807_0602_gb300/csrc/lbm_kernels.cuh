@@ -1133,9 +1133,9 @@ __device__ __forceinline__ void bar_group(int g) {
 // One tile of the march.  `ready` is called once per thread after everything
 // that does not depend on the populations has been loaded (the chained launch
 // waits there for the tiles it reads); NC as in ldp.
-template <typename S, int W, bool G, bool NC, typename Ready>
+template <typename S, int W, bool G, bool NC, bool UNI, typename Ready>
 __device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, const Tile* __restrict__ tiles, int tile,
-                                           int parity, Ready ready) {
+                                           int parity, const Shape& shape, Ready ready) {
     using C = typename Prec<S>::C;
     // FP32 arithmetic never reads f_0 after the pull (the rest population is
     // n_k minus the moving ones), so it stages 16 populations of the collided
@@ -1178,8 +1178,8 @@ __device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, con
         return;
     }
 #else
-    const int nx = rd.nx, ny = rd.ny, pitch = rd.pitch;
-    const unsigned plane = (unsigned)rd.plane;
+    const int nx = UNI ? shape.nx : rd.nx, ny = UNI ? shape.ny : rd.ny, pitch = UNI ? shape.pitch : rd.pitch;
+    const unsigned plane = UNI ? shape.plane : (unsigned)rd.plane;
 #endif
     const Geo geo{nx, rd.cap_x0, rd.cap_x1, rd.y_bot, rd.y_top, rd.mask};
     const S* src = static_cast<const S*>(rd.buf[parity]);
@@ -1357,7 +1357,15 @@ template <typename S, int W, bool G>
 __global__ void __launch_bounds__(2 * W, (kBidirMinBlocks<S, W>)) k_step_bidir(const RunDesc* __restrict__ runs,
                                                                               const Tile* __restrict__ tiles,
                                                                               int parity) {
-    bidir_tile<S, W, G, false>(runs, tiles, blockIdx.x, parity, [] { step_ready(); });
+    bidir_tile<S, W, G, false, false>(runs, tiles, blockIdx.x, parity, Shape{}, [] { step_ready(); });
+}
+
+// The same for runs of one size, given as parameters.
+template <typename S, int W, bool G>
+__global__ void __launch_bounds__(2 * W, (kBidirMinBlocks<S, W>)) k_step_bidir_alike(const RunDesc* __restrict__ runs,
+                                                                                    const Tile* __restrict__ tiles,
+                                                                                    int parity, Shape shape) {
+    bidir_tile<S, W, G, false, true>(runs, tiles, blockIdx.x, parity, shape, [] { step_ready(); });
 }
 
 // ---- two-columns-per-thread variant ---------------------------------------------

@@ -240,8 +240,14 @@ static cudaError_t bidir_smem() {
 
 template <typename S, bool G>
 cudaError_t Step<S, G>::step_bidir(int W, const RunDesc* d_runs, const Tile* d_tiles, int ntiles, int parity,
-                                  cudaStream_t s) {
+                                  const Shape& shape, cudaStream_t s) {
     if (ntiles <= 0) return cudaSuccess;
+    if constexpr (sizeof(typename Prec<S>::C) == 4) {
+        if (shape.nx > 0 && W == 64)
+            return launch_step(k_step_bidir_alike<S, 64, G>, ntiles, 128, s, d_runs, d_tiles, parity, shape);
+        if (shape.nx > 0 && W == 128)
+            return launch_step(k_step_bidir_alike<S, 128, G>, ntiles, 256, s, d_runs, d_tiles, parity, shape);
+    }
     switch (W) {
         case 64: {
             const cudaError_t e = bidir_smem<S, G>();
