@@ -54,10 +54,11 @@ BYTES_PER_NODE = {"f64": 288, "f32": 144, "f16s": 72}
 # 4 x 33)
 TUNE_STEPS = 2000
 KERNELS = ["register", "cp.async", "tma", "pipelined", "split", "l2-prefetch", "smem-staged", "column-pair",
-           "node-tile", "bidirectional", "ring", "bidirectional-jit", "chain"]
+           "node-tile", "bidirectional", "ring", "bidirectional-jit", "chain", "two-step"]
 KERNEL_NAMES = ["k_step", "k_step_async", "k_step_tma", "k_step_pf", "k_step_split", "k_step (L2 prefetch)",
                 "k_step_smem", "k_step_pair", "k_step_tile", "k_step_bidir", "k_step_ring",
-                "k_step_bidir (compiled for the grid)", "k_chain_bidir"]
+                "k_step_bidir (compiled for the grid)", "k_chain_bidir",
+                "k_two_steps"]
 # committed ncu summaries of the step kernel on this workload, by (variant, tile)
 # keyed by (kernel, tile, species): species None for alpha = 4/9, m = 1, else --species
 SPECIES_1_3 = (4.0 / 9.0, 0.8, 1.0, 25.0 / 9.0)

@@ -370,6 +370,11 @@ int lbm_set_tiling(lbm_t* h, int tile_w, int tile_h);
  *                         all its steps up to the next log record as one
  *                         launch (graph_chunk > 0: that many), inside a CUDA
  *                         graph where the log is on and whole.
+ *   LBM_KERNEL_TWO_STEP   LBM_KERNEL_TILE with tile_w 32 and tile_h 6, but four
+ *                         steps at a time are two launches of two steps each
+ *                         (the last step of an lbm_step call or a log interval
+ *                         is always a single one); LBM_F32 and LBM_F16S;
+ *                         nx, ny >= 4.
  * depth is read by LBM_KERNEL_ASYNC, LBM_KERNEL_TMA and LBM_KERNEL_RING and
  * must be 4 for the others.  lbm_set_schedule returns LBM_EINVAL for an unsupported
  * combination, leaving the schedule unchanged. */
@@ -386,6 +391,7 @@ int lbm_set_tiling(lbm_t* h, int tile_w, int tile_h);
 #define LBM_KERNEL_BIDIR 9       /* two thread groups marching away from the tile's middle row */
 #define LBM_KERNEL_RING 10       /* persistent producer/consumer ring of bulk-copied row slots (FP32, FP16S) */
 #define LBM_KERNEL_BIDIR_JIT 11  /* LBM_KERNEL_BIDIR compiled at run time for the handle's grid (one run) */
+#define LBM_KERNEL_TWO_STEP 13   /* node tiles, two steps per launch (FP32, FP16S) */
 #define LBM_KERNEL_CHAIN 12      /* LBM_KERNEL_BIDIR's tiles, many steps chained in one launch (FP64) */
 int lbm_get_schedule(const lbm_t* h, int* tile_w, int* tile_h, int* kernel, int* depth);
 /* The autotuner's finalists (the paper has no counterpart: this reports on the

@@ -56,7 +56,8 @@ struct lbm_s {
                                    // groups marching away from the tile's middle row, 10 persistent
                                    // producer/consumer ring of row slots filled by bulk copies, 11 the
                                    // bidirectional march compiled at run time for the run's grid, 12
-                                   // chained steps over bidirectional tiles (lbm_chain.cuh)
+                                   // chained steps over bidirectional tiles (lbm_chain.cuh), 13 node tiles
+                                   // with two steps per launch
     int* d_queue = nullptr;        // ring kernel: segment counter and finished-CTA counter
     int ring_grid = 0;             // ring kernel: CTAs of the persistent grid
     std::vector<int> chain_tab;    // chained steps (kvar 12): ChainTiles' tables, deps, flags, control words, span
@@ -64,6 +65,9 @@ struct lbm_s {
     int chain_cap = 0;             // tiles these tables have room for
     int chain_grid = 0;            // CTAs of a chained launch
     int chain_rot = 0;             // tiles each step starts further on
+    std::vector<Tile> pair_tiles;  // kvar 13: tiles of the two-step kernel
+    Tile* d_pair_tiles = nullptr;
+    size_t d_pair_cap = 0;
     const void* jit_fn = nullptr;  // kvar 11: the bidirectional march compiled for this run's grid
     std::vector<int2> rows;
     int2* d_rows = nullptr;
@@ -344,7 +348,31 @@ int upload_chain(lbm_t* h, int W, int R) {
     return LBM_OK;
 }
 
+int upload_pair_tiles(lbm_t* h) {
+    h->pair_tiles.clear();
+    for (int r = 0; r < h->nruns; ++r) {
+        const RunDesc& rd = h->runs[r];
+        for (int y0 = 0; y0 < rd.ny; y0 += sc::kPairRows)
+            for (int x0 = 0; x0 < rd.nx; x0 += sc::kPairCols)
+                h->pair_tiles.push_back({r, x0, y0, std::min(y0 + sc::kPairRows, rd.ny)});
+    }
+    const size_t need = h->pair_tiles.size() * sizeof(Tile);
+    if (need > h->d_pair_cap) {   // an old table may still be in use: kept until destroy
+        Tile* p = static_cast<Tile*>(dalloc(h, need));
+        if (!p) return LBM_ENOMEM;
+        h->d_pair_tiles = p;
+        h->d_pair_cap = need;
+    }
+    // upload_tiles synchronises before the vector can change
+    CK(h, cudaMemcpyAsync(h->d_pair_tiles, h->pair_tiles.data(), need, cudaMemcpyHostToDevice, h->stream));
+    return LBM_OK;
+}
+
 int upload_tiles(lbm_t* h, int W, int R) {
+    if (h->kvar == 13) {
+        const int rc = upload_pair_tiles(h);
+        if (rc) return rc;
+    }
     if (h->kvar == 12) {
         const int rc = upload_chain(h, W, R);
         if (rc) return rc;
@@ -430,7 +458,7 @@ cudaError_t issue_step(lbm_t* h, int parity, cudaStream_t s) {
         return dispatch_step(h, [&](auto L) { return L.step_pair(W, h->d_runs, h->d_tiles, nt, parity, s); });
     if (h->kvar == 9)
         return dispatch_step(h, [&](auto L) { return L.step_bidir(W, h->d_runs, h->d_tiles, nt, parity, h->shape, s); });
-    if (h->kvar == 8)
+    if (h->kvar == 8 || h->kvar == 13)
         return dispatch_step(h,
                              [&](auto L) { return L.step_tile(W, h->tile_h, h->d_runs, h->d_tiles, nt, parity, s); });
     if (h->kvar == 10)
@@ -457,8 +485,33 @@ cudaError_t issue_step(lbm_t* h, int parity, cudaStream_t s) {
     return dispatch_step(h, [&](auto L) { return L.step(W, h->d_runs, h->d_tiles, nt, parity, s); });
 }
 
+// Issues n steps on stream s.  The two-step kernel leaves the state of t + 2 in
+// the buffer of t + 1, so its launches come in pairs (four steps), and the
+// last step is a single one: both buffers then hold the states of the last
+// two times, as after single steps.
+cudaError_t issue_steps(lbm_t* h, int parity, int n, cudaStream_t s) {
+    if (chained(h)) return issue_chain(h, parity, n, s);
+    int j = 0;
+    cudaError_t e = cudaSuccess;
+    if (h->kvar == 13) {
+        for (; j + 4 < n && e == cudaSuccess; j += 4)
+            for (int b = 0; b < 2 && e == cudaSuccess; ++b)
+                e = dispatch_step(h, [&](auto L) {
+                    return L.two_steps(h->d_runs, h->d_pair_tiles, (int)h->pair_tiles.size(), parity ^ b, s);
+                });
+    }
+    for (; j < n && e == cudaSuccess; ++j) e = issue_step(h, (parity + j) & 1, s);
+    return e;
+}
+
 bool schedule_ok(const lbm_t* h, int W, int R, int kvar, int depth) {
-    if (R < 1 || kvar < 0 || kvar > 12) return false;
+    if (R < 1 || kvar < 0 || kvar > 13) return false;
+    if (kvar == 13) {   // node tiles, two steps per launch: FP32 arithmetic, periodic images up to three nodes away
+        if (h->precision == LBM_F64 || W != 32 || R != 6) return false;
+        for (const RunDesc& rd : h->runs)
+            if (rd.ny < 4) return false;
+        kvar = 8;
+    }
     if (kvar == 12) {   // chained bidirectional tiles: FP64, and the march's tilings
         if (h->precision != LBM_F64) return false;
         kvar = 9;
@@ -539,9 +592,7 @@ int get_graph(lbm_t* h, int parity, int steps, int with_log, cudaGraphExec_t* ou
     cudaGraph_t g = nullptr;
     CK(h, cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
-    if (chained(h)) e = issue_chain(h, parity, steps, h->cap_stream);
-    else
-        for (int j = 0; j < steps && e == cudaSuccess; ++j) e = issue_step(h, (parity + j) & 1, h->cap_stream);
+    e = issue_steps(h, parity, steps, h->cap_stream);
     if (e == cudaSuccess && with_log) e = issue_log(h, (parity + steps) & 1, h->cap_stream);
     cudaError_t e2 = cudaStreamEndCapture(h->cap_stream, &g);
     if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -597,10 +648,8 @@ int advance(lbm_t* h, int64_t n) {
             if (le > 0) h->nlog += 1;
         } else {
             NvtxRange range("lbm steps");
-            for (int64_t j = 0; j < m; ++j) {
-                CK(h, issue_step(h, (int)(h->t & 1), h->stream));
-                h->t += 1;
-            }
+            CK(h, issue_steps(h, (int)(h->t & 1), (int)m, h->stream));
+            h->t += m;
             if (le > 0 && h->t % le == 0) {
                 CK(h, issue_log(h, (int)(h->t & 1), h->stream));
                 h->nlog += 1;
@@ -647,28 +696,31 @@ struct Sched {
 
 // The schedule of a handle that nobody has chosen one for, by the size of its
 // runs.  Measured on a GB300, us per step:
-//   - FP32 and FP16S up to 250 000 nodes: one node per thread (32 x 6 tiles).
-//     Every load of a tile is in flight at once, and small grids are bound by
-//     that latency: 256 x 32 2.4 (bidirectional 3.3, staged march 128 x 4 8.0),
-//     1024 x 66 4.0 (4.6, 8.2); equal at 274 000 nodes (4095 x 67 with two
-//     masses 8.6, 8.7, 11.8), then behind: 16 droplets of 256 x 128 19.4
-//     (16.2, 23.3), 8192 x 160 43 (36.8, 43).
+//   - FP32 and FP16S up to 130 000 nodes: one node per thread (32 x 6 tiles) and
+//     two steps per launch. Every load of a tile is in flight at once, and small
+//     grids are bound by that latency and by the launch boundaries: 256 x 32
+//     2.1 (single node-tile steps 2.35, bidirectional 2.9, staged march 128 x 4
+//     8.0), 1024 x 66 3.0 (4.0, 4.1, 8.2), 2000 x 66 5.1 (5.4, 5.6).
+//   - up to 250 000 nodes single node-tile steps: equal to the bidirectional
+//     march at 274 000 (4095 x 67 with two masses 8.6, 8.7, staged 11.8), then
+//     behind: 16 droplets of 256 x 128 19.4 (16.2, 23.3), 8192 x 160 43 (36.0, 43).
 //   - larger ones: the bidirectional march, tiles of 12 rows or fewer so that
-//     they fill whole waves of resident CTAs: 8192 x 160 36.8, FP16S 31.7
-//     (staged march 43.0, 35.0), 256 droplets 274 (308), 64 uneven capillaries
+//     they fill whole waves of resident CTAs: 8192 x 160 36.7, FP16S 29.8
+//     (staged march 43.0, 35.0), 256 droplets 268 (308), 64 uneven capillaries
 //     488 (531).
 //   - FP64 from 30 000 nodes on: chained steps, tiles low enough for about 1000
-//     of them: 2048 x 130 154 (staged march 209), nine 128 x 80 droplets 88
-//     (164); below that (256 x 32: 22, 83) the bidirectional march with tiles
-//     of two rows.
+//     of them: 2048 x 130 103 (bidirectional 124, staged march 180), nine
+//     128 x 80 droplets 54 (72, 155); below that (256 x 32: 20.5, chained 26)
+//     the bidirectional march with tiles of two rows.
 Sched default_schedule(lbm_t* h) {
     double nodes = 0.0, strip_rows = 0.0;
-    int maxny = 1, minnx = 1 << 30;
+    int maxny = 1, minnx = 1 << 30, minny = 1 << 30;
     for (const RunDesc& rd : h->runs) {
         nodes += rd.nodes;
         strip_rows += (double)((rd.nx + 61) / 62) * rd.ny;
         maxny = std::max(maxny, rd.ny);
         minnx = std::min(minnx, rd.nx);
+        minny = std::min(minny, rd.ny);
     }
     if (h->precision == LBM_F64) {
         if (nodes < 30000) return {64, std::min(2, maxny), 9, 4};
@@ -676,6 +728,7 @@ Sched default_schedule(lbm_t* h) {
         const int R = std::max(1, std::min({(int)(strip_rows / 900.0), 16, maxny}));
         return {64, R > 1 ? R & ~1 : R, 12, 4};
     }
+    if (nodes <= 130000 && minnx >= 4 && minny >= 4) return {32, 6, 13, 4};
     if (nodes <= 250000 && minnx >= 4) return {32, 6, 8, 4};
     int R = std::min(12, maxny), per_sm = 0, dev = 0, sms = 0;
     if (dispatch_step(h, [&](auto L) { return L.bidir_ctas_per_sm(64, &per_sm); }) == cudaSuccess && per_sm > 0 &&

@@ -88,6 +88,9 @@ constexpr int kNoFront = 0x7f7f7f7f;
 // collided columns per strip of the persistent ring kernel (LBM_KERNEL_RING)
 constexpr int kRingWc = 120;
 
+// stored nodes per tile of the two-step kernel
+constexpr int kPairCols = 26, kPairRows = 10;
+
 // opt-in shared memory per CTA on sm_103a (227 KB)
 constexpr size_t kMaxSmemPerCta = 232448;
 
@@ -183,6 +186,8 @@ struct Step {
                                  int parity, uint32_t* err, cudaStream_t s);
     // resident CTAs per SM of that kernel (0 if not available)
     static cudaError_t ring_ctas_per_sm(int D, int* out);
+    // two steps in one launch (FP32 and FP16S storage; tiles of kPairCols x kPairRows nodes)
+    static cudaError_t two_steps(const RunDesc* d_runs, const Tile* d_tiles, int ntiles, int parity, cudaStream_t s);
     // chained steps (lbm_chain.cuh, FP64): nsteps steps in one launch of `grid`
     // CTAs over tiles of the bidirectional march of W = 64 threads per group
     static cudaError_t chain(const RunDesc* d_runs, const ChainTiles& ct, int nsteps, int parity, int rot, int grid,

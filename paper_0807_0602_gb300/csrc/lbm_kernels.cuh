@@ -1657,6 +1657,89 @@ __global__ void __launch_bounds__(W * TY, (kTileMinBlocks<S, W, TY>)) k_step_til
     node_tile<S, W, TY, G, false>(runs, tiles, blockIdx.x, parity, [] { step_ready(); });
 }
 
+// ---- two steps per launch on small grids ----------------------------------------
+// On a small grid a step is the launch boundary (the step before must be
+// complete and visible: about a microsecond) and one node's chain of latencies;
+// the SMs are mostly idle.  A CTA of 32 x 16 threads here takes 26 x 10 nodes
+// through two steps: it pulls and collides the nodes around them too (32 x 16
+// pulled, 30 x 14 collided, 28 x 12 pulled again, 26 x 10 stored), with the
+// populations between the steps in shared memory, rounded to the storage type
+// as memory would.  Half the work is redundant and half the boundaries are
+// gone.  Reads buf[parity], writes the state two steps later to the other
+// buffer.  FP32 and FP16S; nx, ny >= 4.  GB300, us per step against single
+// node-tile steps: 256x32 2.12 / 2.35, 512x66 2.25 / 2.83, 1024x66 3.03 / 3.99,
+// 2000x66 5.10 / 5.43.
+template <typename S> __device__ __forceinline__ float stored(float v, float sh);
+template <> __device__ __forceinline__ float stored<float>(float v, float) { return v; }
+template <> __device__ __forceinline__ float stored<__half>(float v, float sh) {
+    return dec(__float2half_rn(__fsub_rn(v, sh)), sh);
+}
+
+template <typename S, bool G>
+__global__ void __launch_bounds__(512, 2) k_two_steps(const RunDesc* __restrict__ runs, const Tile* __restrict__ tiles,
+                                                      int parity) {
+    constexpr int W = 32, TY = 16;
+    __shared__ float P[18][TY][W];
+    __shared__ float sa[TY][2][W], sb[TY][2][W];
+    const Tile tl = tiles[blockIdx.x];
+    const RunDesc& rd = runs[tl.run];
+    const bool tile_ok = step_tile_ok(tl, rd);
+    const int nx = rd.nx, ny = rd.ny, pitch = rd.pitch;
+    const unsigned plane = (unsigned)rd.plane;
+    const S* src = static_cast<const S*>(rd.buf[parity]);
+    S* dst = static_cast<S*>(rd.buf[parity ^ 1]);
+    StepCtx<S, G> cx;
+    cx.load(rd);
+    const int tx = threadIdx.x % W, ty = threadIdx.x / W;
+    const int x = tl.x0 - 3 + tx, y = tl.y0 - 3 + ty;   // unwrapped
+    const int xe = min(tl.x0 + kPairCols, nx), ye = tl.y1;
+    const bool act = tile_ok && x <= xe + 2 && y <= ye + 2;
+    const int xw = !act ? 0 : (x < 0 ? x + nx : (x >= nx ? x - nx : x));
+    const RowIdx q = rows_of(act ? (y < 0 ? y + ny : (y >= ny ? y - ny : y)) : 0, ny);
+    const int xm = xw == 0 ? nx - 1 : xw - 1, xp = xw == nx - 1 ? 0 : xw + 1;
+    const Geo geo{nx, rd.cap_x0, rd.cap_x1, rd.y_bot, rd.y_top, rd.mask};
+    const unsigned m = act ? nbr_solid(geo, xm, xw, xp, q.rm, q.rw, q.rp) : 0;
+    const bool fluid = act && !SOL(m, 0, 0);
+    float f[2][9];
+    float nA = 0.f, nB = 0.f;
+    step_ready();
+    if (fluid) {
+        const unsigned bw = (unsigned)(q.rw * pitch), bm = (unsigned)(q.rm * pitch), bp = (unsigned)(q.rp * pitch);
+        pull_node<S, false>(src, plane, bw + xw, bw + xm, bw + xp, bm + xw, bp + xw, bm + xm, bm + xp, bp + xm, bp + xp,
+                            m, cx.sh, f);
+        nA = dens9(f[0]);
+        nB = dens9(f[1]);
+    }
+    sa[ty][0][tx] = nA;
+    sa[ty][1][tx] = nB;
+    __syncthreads();
+    if (fluid && tx >= 1 && tx < W - 1 && ty >= 1 && ty < TY - 1 && x <= xe + 1 && y <= ye + 1) {
+        NodeState<S> ns;
+        node_state<S, W>(cx, f, m, sa, ty - 1, ty, ty + 1, tx, ns);
+        float fn[2][9];
+        relax<S>(cx, f, ns, fn);
+#pragma unroll
+        for (int i = 0; i < 18; ++i) P[i][ty][tx] = stored<S>(fn[i / 9][i % 9], cx.sh.v[i / 9][grp(i % 9)]);
+    }
+    __syncthreads();
+    nA = nB = 0.f;
+    if (fluid && tx >= 2 && tx < W - 2 && ty >= 2 && ty < TY - 2 && x <= xe && y <= ye) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int i = 0; i < 9; ++i)
+                f[k][i] = SOL(m, -cyo(i), -cxo(i)) ? P[9 * k + opp(i)][ty][tx] : P[9 * k + i][ty - cyo(i)][tx - cxo(i)];
+        nA = dens9(f[0]);
+        nB = dens9(f[1]);
+    }
+    sb[ty][0][tx] = nA;
+    sb[ty][1][tx] = nB;
+    __syncthreads();
+    if (fluid && tx >= 3 && tx < W - 3 && ty >= 3 && ty < TY - 3 && x < xe && y < ye)
+        collide_any<S, W, 0>(cx, f, m, sb, ty - 1, ty, ty + 1, tx, dst, plane, (unsigned)(q.rw * pitch + xw),
+                             MomOut{nullptr, nullptr, 0}, 0, ghost_r(xw, nx), ghost_l(xw, nx));
+}
+
 // ---- software-pipelined staged variant ---------------------------------------
 // k_step_smem's march with the loads of row r + 2 issued (into raw
 // registers) before row r is collided, and decoded (densities into the ring,

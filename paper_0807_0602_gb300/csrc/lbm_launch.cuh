@@ -316,6 +316,16 @@ cudaError_t Step<S, G>::bidir_ctas_per_sm(int W, int* out) {
 }
 
 template <typename S, bool G>
+cudaError_t Step<S, G>::two_steps(const RunDesc* d_runs, const Tile* d_tiles, int ntiles, int parity, cudaStream_t s) {
+    if constexpr (sizeof(S) == 8) {
+        return cudaErrorInvalidValue;   // FP64 is bound by its pipe: no redundant work
+    } else {
+        if (ntiles <= 0) return cudaSuccess;
+        return launch_step(k_two_steps<S, G>, ntiles, 512, s, d_runs, d_tiles, parity);
+    }
+}
+
+template <typename S, bool G>
 cudaError_t Step<S, G>::chain(const RunDesc* d_runs, const ChainTiles& ct, int nsteps, int parity, int rot, int grid,
                               uint32_t* err, cudaStream_t s) {
     if constexpr (sizeof(S) != 8) {

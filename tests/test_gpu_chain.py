@@ -89,7 +89,8 @@ def test_chain_is_refused_outside_fp64_and_its_tilings():
 
 
 # grids on both sides of the sizes at which the starting schedule changes
-@pytest.mark.parametrize("prec,nx,ny", [("f32", 33, 7), ("f32", 3, 5), ("f32", 300, 40), ("f32", 2500, 100),
+@pytest.mark.parametrize("prec,nx,ny", [("f32", 33, 7), ("f32", 3, 5), ("f32", 300, 40), ("f32", 1300, 100),
+                                        ("f32", 1301, 100), ("f32", 2500, 100),
                                         ("f32", 2501, 100), ("f32", 1300, 700), ("f16s", 300, 40),
                                         ("f16s", 2501, 100), ("f64", 100, 40), ("f64", 300, 99), ("f64", 300, 101)])
 def test_starting_schedule_gives_the_same_bits(prec, nx, ny):
@@ -124,3 +125,33 @@ def test_checkpoint_of_a_starting_schedule_loads(tmp_path):
             with Lat.load(str(tmp_path / prec)) as b:
                 b.step(8)
                 assert np.array_equal(a.populations(), b.populations())
+
+
+# less than a tile, exact tiles, one column or row more, wraps on every side
+@pytest.mark.parametrize("nx,ny,kind", [(4, 4, "box"), (26, 10, "box"), (27, 11, "cap"), (25, 9, "mask"),
+                                        (53, 31, "mask"), (130, 20, "cap")])
+@pytest.mark.parametrize("prec,ratio", [("f32", False), ("f32", True), ("f16s", False)])
+def test_two_steps_per_launch_equal_single_steps(nx, ny, kind, prec, ratio):
+    run = _run(nx, ny, kind, ratio)
+    kw = dict(precision=prec, rho_ref=(1.0, 1.0), log_every=11, log_capacity=8)
+    with Lattice(run, tile=(32, 6), kernel=(13, 4), **kw) as a, Lattice(run, tile=(128, 4), kernel=(6, 4), **kw) as b:
+        for n in (1, 4, 5, 6, 9, 20):     # both parities at the start, whole log intervals and parts
+            a.step(n)
+            b.step(n)
+            assert np.array_equal(a.populations().view(np.uint8), b.populations().view(np.uint8))
+            for p, q in zip(a.velocity(), b.velocity()):   # reads the state of the step before
+                assert np.array_equal(p, q)
+        assert np.array_equal(a.log(), b.log(), equal_nan=True)
+
+
+def test_two_step_tilings_are_validated():
+    from paper_0807_0602_gb300 import _lib as L
+    with Lattice(_run(64, 18, "cap"), precision="f32") as lat:
+        before = lat.schedule
+        for bad in ((64, 6, 13, 4), (32, 14, 13, 4), (32, 6, 13, 3)):
+            with pytest.raises(L.LbmError):
+                lat.schedule = bad
+        assert lat.schedule == before
+    with Lattice(_run(64, 3, "box"), precision="f32") as lat:   # fewer than four rows
+        with pytest.raises(L.LbmError):
+            lat.schedule = (32, 6, 13, 4)
