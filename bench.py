@@ -63,6 +63,8 @@ KERNEL_NAMES = ["k_step", "k_step_async", "k_step_tma", "k_step_pf", "k_step_spl
 # keyed by (kernel, tile, species): species None for alpha = 4/9, m = 1, else --species
 SPECIES_1_3 = (4.0 / 9.0, 0.8, 1.0, 25.0 / 9.0)
 PROFILES = {
+    (11, (128, 18), None, "f32"): os.path.join(ROOT, "profiles",
+                                               "k_step_bidir_jit_tile128x18_f32_capillary_8192x160.txt"),
     (11, (64, 18), None, "f32"): os.path.join(ROOT, "profiles", "k_step_bidir_jit_tile64x18_f32_capillary_8192x160.txt"),
     (11, (64, 9), None, "f32"): os.path.join(ROOT, "profiles", "k_step_bidir_jit_tile64x9_f32_capillary_8192x160.txt"),
     (9, (64, 18), None, "f32"): os.path.join(ROOT, "profiles", "k_step_bidir_tile64x18_f32_capillary_8192x160.txt"),
@@ -72,19 +74,28 @@ PROFILES = {
     (11, (64, 9), None, "f16s"): os.path.join(ROOT, "profiles", "k_step_bidir_jit_tile64x9_f16s_capillary_8192x160.txt"),
     (11, (64, 18), None, "f16s"): os.path.join(ROOT, "profiles",
                                                "k_step_bidir_jit_tile64x18_f16s_capillary_8192x160.txt"),
+    (9, (64, 8), None, "f16s"): os.path.join(ROOT, "profiles", "k_step_bidir_tile64x8_f16s_capillary_8192x160.txt"),
     (9, (64, 9), None, "f16s"): os.path.join(ROOT, "profiles", "k_step_bidir_tile64x9_f16s_capillary_8192x160.txt"),
     (6, (128, 4), None, "f64"): os.path.join(ROOT, "profiles", "k_step_smem_tile128x4_f64_capillary_8192x160.txt"),
     (0, (128, 4), None, "f64"): os.path.join(ROOT, "profiles",
                                              "k_step_register_tile128x4_f64_capillary_8192x160.txt"),
+    (9, (64, 8), None, "f64"): os.path.join(ROOT, "profiles", "k_step_bidir_tile64x8_f64_capillary_8192x160.txt"),
     (11, (64, 8), None, "f64"): os.path.join(ROOT, "profiles", "k_step_bidir_jit_tile64x8_f64_capillary_8192x160.txt"),
     (9, (64, 18), SPECIES_1_3, "f32"): os.path.join(ROOT, "profiles",
                                                     "k_step_bidir_species_tile64x18_f32_capillary_8192x160.txt"),
     (11, (64, 18), SPECIES_1_3, "f32"): os.path.join(ROOT, "profiles",
                                                      "k_step_bidir_jit_species_tile64x18_f32_capillary_8192x160.txt"),
 }
+# the FP64 kernels whose instruction counts are committed
+FP64_PROFILES = {
+    (6, (128, 4)): PROFILES[(6, (128, 4), None, "f64")],
+    (0, (128, 4)): PROFILES[(0, (128, 4), None, "f64")],
+    (9, (64, 8)): PROFILES[(9, (64, 8), None, "f64")],
+    (12, (64, 16)): os.path.join(ROOT, "profiles", "k_chain_bidir_tile64x16_f64_capillary_8192x160.txt"),
+}
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_0807_0602_gb300", "csrc", f)
-                  for f in ("lbm_kernels.cuh", "lbm_ring.cuh", "lbm_launch.cuh", "kernels_f32.cu",
-                            "kernels_gen_f32.cu", "lbm_device.h", "lbm_jit.cu")]
+                  for f in ("lbm_kernels.cuh", "lbm_exact.h", "lbm_chain.cuh", "lbm_ring.cuh", "lbm_launch.cuh",
+                            "kernels_f32.cu", "kernels_gen_f32.cu", "lbm_device.h", "lbm_jit.cu")]
 
 
 # (alpha_A, alpha_B, m_A, m_B) of --species, or None for alpha = 4/9, m = 1
@@ -401,15 +412,16 @@ def select_schedule(lat, stream, flush, steps: int = 24, log_every: int = 50):
                     "the fastest median kept"}
 
 
-def fp64_ops_per_node():
+def fp64_ops_per_node(kvar: int, tile):
     """FP64 instructions per node of the step (DADD + DMUL + DFMA thread
-    instructions, from the committed FP64 ncu summary), or None when the
-    kernel sources changed since.  Every FP64 step kernel evaluates the same
-    canonical arithmetic, so the count holds for each of them."""
-    path = PROFILES[(6, (128, 4), None, "f64")]
+    instructions, from the committed ncu summary of this FP64 kernel and
+    tile), or None when there is none or the kernel sources changed since.
+    The kernels differ: the bidirectional and chained marches share the
+    products w n, and taller tiles pull fewer halo rows."""
+    path = FP64_PROFILES.get((int(kvar), (int(tile[0]), int(tile[1]))))
     try:
         kv = {}
-        with open(path) as fh:
+        with open(path or "") as fh:
             for line in fh:
                 if ":" in line and not line.startswith("#"):
                     k, v = line.split(":", 1)
@@ -465,7 +477,7 @@ def measure_precision(stream, dev, precision: str, steps: int = 200):
         with torch.cuda.stream(stream):
             L.check(lib.lbm_selftest_fp64_rate(ctypes.byref(rate), ctypes.c_void_p(stream.cuda_stream)),
                     "lbm_selftest_fp64_rate")
-        ops = fp64_ops_per_node()
+        ops = fp64_ops_per_node(sched[2], sched[:2])
         fp64 = {"bound": "fp64 pipe", "unit": "FP64 instructions/s",
                 "peak": rate.value / 2.0, "peak_source": "measured: lbm_selftest_fp64_rate (DFMA chains, "
                                                          "2 flops each) / 2 = DFMA instructions per second",
