@@ -424,12 +424,14 @@ sc::LogCtl logctl(lbm_t* h) {
 
 // Issues n chained steps on stream s (parity = t & 1 of the first).
 cudaError_t issue_chain(lbm_t* h, int parity, int n, cudaStream_t s) {
-    const int nt = (int)h->tiles.size();
+    // a single step has nothing to chain: the bidirectional march takes the same tiles
+    if (n == 1)
+        return dispatch_step(h, [&](auto L) {
+            return L.step_bidir(64, h->d_runs, h->d_tiles, (int)h->tiles.size(), parity, h->shape, s);
+        });
     const sc::ChainTiles ct = chain_tables(h);
-    // a single step has nothing to chain: no more CTAs than tiles
-    const int grid = n == 1 ? std::min(h->chain_grid, nt) : h->chain_grid;
     return dispatch_step(h, [&](auto L) {
-        return L.chain(h->d_runs, ct, n, parity, h->chain_rot, grid, h->d_err, s);
+        return L.chain(h->d_runs, ct, n, parity, h->chain_rot, h->chain_grid, h->d_err, s);
     });
 }
 
