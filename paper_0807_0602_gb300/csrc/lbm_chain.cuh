@@ -19,8 +19,8 @@
 // Where it pays: the FP64 step is bound by the FP64 pipe, so a tile is long (some
 // 20 us for 4 rows) and a grid of a few hundred thousand nodes is one or two
 // waves of them; launched step by step, most SMs idle in the last wave.  GB300,
-// us per step, single steps (best tiling) / chained: 2048 x 130 173 / 154,
-// nine 128 x 80 droplets 111 / 88, 256 x 32 22 / 29 (too few tiles: the flags'
+// us per step, single steps (best tiling) / chained: 2048 x 130 124 / 103,
+// nine 128 x 80 droplets 72 / 54, 256 x 32 20.5 / 26 (too few tiles: the flags'
 // round trips through L2 cost more than launches).  FP32 and FP16S keep single
 // steps: an acquire drops the SM's L1 lines, which their shifted loads live on
 // (64 uneven capillaries FP32: 506 single, 553 chained; 8192 x 160: 37.4, 37.7).

@@ -1240,6 +1240,8 @@ __device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, con
     // and no wrap in y.  They need neither the solid test nor the row and
     // column wraps: columns -1 and nx are read from the ghost columns.  Most
     // rows are plain; the longest run of them in this tile is [pl0, pl0 + pln).
+    // 20.8 -> 18.1 warp instructions per node (FP32 64x9), FP16S 8192x160 35.5 ->
+    // 29.8 us, FP32, bound by the loads in flight, 38.4 -> 36.7.
     int pl0 = max(1, y0 - 1), pln = max(0, min(ny - 2, y1) + 1 - pl0);
     if (geo.mask || nx < 4) pln = 0;
     if ((geo.cx0 <= tl.x0 + sc.ncols + 1 && geo.cx1 > tl.x0 - 2) || tl.x0 == 0 || tl.x0 + sc.ncols == nx) {
