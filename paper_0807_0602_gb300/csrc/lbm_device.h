@@ -101,6 +101,37 @@ struct Tile {
     int run, x0, y0, y1;
 };
 
+// Longest run [first, first + count) of plain rows among the rows y0 - 1 .. y1
+// that the bidirectional march pulls for a tile: no wrap in y, and no solid
+// among the 3x3 neighbours of any column it pulls.  Those are the ncols
+// collided columns and one more on each side, so the neighbours are
+// x0 - 2 .. x0 + ncols + 1.  A strip whose neighbours wrap in x (the first, the
+// last, and the one before a last strip of a single column) counts as next to
+// the plates wherever they are: few strips, and they lose a few rows at most.
+__host__ __device__ inline void plain_rows(const Tile& tl, int ncols, int nx, int ny, int cap_x0, int cap_x1,
+                                           int y_bot, int y_top, bool mask, int& first, int& count) {
+    const int lo = tl.x0 - 2, hi = tl.x0 + ncols + 1;
+    const int top = ny - 2 < tl.y1 ? ny - 2 : tl.y1;
+    first = tl.y0 - 1 > 1 ? tl.y0 - 1 : 1;
+    count = top + 1 > first ? top + 1 - first : 0;
+    if (mask || nx < 4) count = 0;   // (a mask may be solid anywhere; ghost columns need nx >= 4)
+    if ((cap_x0 <= hi && cap_x1 > lo) || lo < 0 || hi >= nx) {
+        for (int p = 0; p < 2; ++p) {
+            const int y = p ? y_top : y_bot;
+            if (y < 0) continue;
+            // keep the longer side of the rows y - 1 .. y + 1
+            const int a = y - 1 - first, b = first + count - (y + 2);
+            if (a >= count || b >= count) continue;   // outside
+            if (a >= b) {
+                count = a > 0 ? a : 0;
+            } else {
+                first = y + 2;
+                count = b > 0 ? b : 0;
+            }
+        }
+    }
+}
+
 // Control words of a chained launch, all zero before it and after it.
 struct ChainCtl {
     int next;      // next item

@@ -1236,29 +1236,13 @@ __device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, con
         put_dens(slot(grp_d, k), nA, nB);
     };
 
-    // Plain rows: no solid among the 3x3 neighbours of any column of the strip
-    // and no wrap in y.  They need neither the solid test nor the row and
-    // column wraps: columns -1 and nx are read from the ghost columns.  Most
-    // rows are plain; the longest run of them in this tile is [pl0, pl0 + pln).
+    // Plain rows (plain_rows) need neither the solid test nor the row and column
+    // wraps: columns -1 and nx are read from the ghost columns.  Most rows are
+    // plain; the longest run of them in this tile is [pl0, pl0 + pln).
     // 20.8 -> 18.1 warp instructions per node (FP32 64x9), FP16S 8192x160 35.5 ->
     // 29.8 us, FP32, bound by the loads in flight, 38.4 -> 36.7.
-    int pl0 = max(1, y0 - 1), pln = max(0, min(ny - 2, y1) + 1 - pl0);
-    if (geo.mask || nx < 4) pln = 0;
-    if ((geo.cx0 <= tl.x0 + sc.ncols + 1 && geo.cx1 > tl.x0 - 2) || tl.x0 == 0 || tl.x0 + sc.ncols == nx) {
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            const int y = p ? geo.yt : geo.yb;
-            if (y < 0) continue;
-            // keep the longer side of the rows y - 1 .. y + 1
-            const int a = y - 1 - pl0, b = pl0 + pln - (y + 2);
-            if (a >= pln || b >= pln) continue;   // outside
-            if (a >= b) pln = max(a, 0);
-            else {
-                pl0 = y + 2;
-                pln = max(b, 0);
-            }
-        }
-    }
+    int pl0, pln;
+    plain_rows(tl, sc.ncols, nx, ny, geo.cx0, geo.cx1, geo.yb, geo.yt, geo.mask != nullptr, pl0, pln);
     // byte offset of this thread's column in row 0, from LBM_COL0 columns
     // before column 0
     const char* const usrc = reinterpret_cast<const char*>(src - LBM_COL0);
