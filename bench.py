@@ -94,8 +94,8 @@ FP64_PROFILES = {
     (12, (64, 16)): os.path.join(ROOT, "profiles", "k_chain_bidir_tile64x16_f64_capillary_8192x160.txt"),
 }
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_0807_0602_gb300", "csrc", f)
-                  for f in ("lbm_kernels.cuh", "lbm_exact.h", "lbm_chain.cuh", "lbm_ring.cuh", "lbm_launch.cuh",
-                            "kernels_f32.cu", "kernels_gen_f32.cu", "lbm_device.h", "lbm_jit.cu")]
+                  for f in ("lbm_kernels.cuh", "lbm_exact.h", "lbm_chain.cuh", "lbm_chain_items.h", "lbm_ring.cuh",
+                            "lbm_launch.cuh", "kernels_f32.cu", "kernels_gen_f32.cu", "lbm_device.h", "lbm_jit.cu")]
 
 
 # (alpha_A, alpha_B, m_A, m_B) of --species, or None for alpha = 4/9, m = 1

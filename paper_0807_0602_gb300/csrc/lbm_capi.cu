@@ -10,6 +10,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "lbm.h"
+#include "lbm_chain_items.h"
 #include "lbm_device.h"
 #include "lbm_jit.h"
 
@@ -422,17 +423,26 @@ sc::LogCtl logctl(lbm_t* h) {
     return lc;
 }
 
-// Issues n chained steps on stream s (parity = t & 1 of the first).
-cudaError_t issue_chain(lbm_t* h, int parity, int n, cudaStream_t s) {
-    // a single step has nothing to chain: the bidirectional march takes the same tiles
-    if (n == 1)
-        return dispatch_step(h, [&](auto L) {
-            return L.step_bidir(64, h->d_runs, h->d_tiles, (int)h->tiles.size(), parity, h->shape, s);
-        });
+// Issues n chained steps on stream s (parity = t & 1 of the first), as many to
+// a launch as its item numbers allow.
+cudaError_t issue_chain(lbm_t* h, int parity, int64_t n, cudaStream_t s) {
     const sc::ChainTiles ct = chain_tables(h);
-    return dispatch_step(h, [&](auto L) {
-        return L.chain(h->d_runs, ct, n, parity, h->chain_rot, h->chain_grid, h->d_err, s);
-    });
+    cudaError_t e = cudaSuccess;
+    while (n > 0 && e == cudaSuccess) {
+        const int m = (int)sc::chain_launch_steps(n, ct.ntiles);
+        // a single step has nothing to chain: the bidirectional march takes the same tiles
+        if (m == 1)
+            e = dispatch_step(h, [&](auto L) {
+                return L.step_bidir(64, h->d_runs, h->d_tiles, (int)h->tiles.size(), parity, h->shape, s);
+            });
+        else
+            e = dispatch_step(h, [&](auto L) {
+                return L.chain(h->d_runs, ct, m, parity, h->chain_rot, h->chain_grid, h->d_err, s);
+            });
+        parity ^= m & 1;
+        n -= m;
+    }
+    return e;
 }
 
 bool chained(const lbm_t* h) { return h->kvar == 12; }
@@ -630,11 +640,10 @@ int advance(lbm_t* h, int64_t n) {
         if (le > 0) m = std::min<int64_t>(n, le - (h->t % le));
         else m = std::min<int64_t>(n, chunk);
         if (chained(h) && (le == 0 || !graphs || m != le)) {
-            // one launch for all of them (with the log on and whole chunks: within their graph)
+            // chained launches for all of them (with the log on and whole intervals: within their graph)
             NvtxRange range("lbm chained steps");
-            const int64_t most = std::max<int64_t>(1, (1 << 30) / (int64_t)h->tiles.size());   // 32-bit item numbers
-            m = std::min(le > 0 ? m : (h->opt.graph_chunk > 0 ? m : n), most);
-            CK(h, issue_chain(h, (int)(h->t & 1), (int)m, h->stream));
+            if (le == 0 && h->opt.graph_chunk <= 0) m = n;
+            CK(h, issue_chain(h, (int)(h->t & 1), m, h->stream));
             h->t += m;
             if (le > 0 && h->t % le == 0) {
                 CK(h, issue_log(h, (int)(h->t & 1), h->stream));

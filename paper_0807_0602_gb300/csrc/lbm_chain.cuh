@@ -31,6 +31,7 @@
 // read-only path, because other SMs write them within the launch.
 #pragma once
 
+#include "lbm_chain_items.h"
 #include "lbm_kernels.cuh"
 
 namespace sc {
@@ -49,15 +50,15 @@ __device__ __forceinline__ int ld_relaxed(const int* p) {
     return v;
 }
 
-// Tile of item `item` (-1 after the last step) and its step.
 __device__ __forceinline__ int chain_item(const ChainTiles& ct, int item, int nsteps, int rot, int& step) {
-    step = item / ct.ntiles;
-    if (step >= nsteps) return -1;
-    const int i = item - step * ct.ntiles;
-    const int2 sp = __ldg(&ct.span[i]);
-    // the run's list rotated by rot tiles per step (rot < 2^10, the list < 2^20: no overflow)
-    const unsigned off = (unsigned)(step % sp.y) * (unsigned)min(rot, sp.y) + (unsigned)(i - sp.x);
-    return sp.x + (int)(off % (unsigned)sp.y);
+    return chain_item_tile(
+        item, ct.ntiles, nsteps, rot,
+        [&](int i, int& first, int& count) {
+            const int2 sp = __ldg(&ct.span[i]);
+            first = sp.x;
+            count = sp.y;
+        },
+        step);
 }
 
 // tile_fn(tile, parity, ready): advances one tile; calls ready() from every
