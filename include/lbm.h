@@ -463,6 +463,15 @@ int lbm_mass_noalloc(const lbm_geometry* g, int precision, const void* populatio
  * cudaStream_t, NULL = default) and allocates and frees 4 bytes. */
 int lbm_selftest_wait_timeout(long long cycles, void* stream);
 
+/* The same for the waits of a chained launch (LBM_KERNEL_CHAIN): launches its
+ * item loop over tiles that wait for a flag which nothing sets, each wait
+ * giving up after `cycles`, and then, with the control words and flags that
+ * this launch left behind, over tiles that wait for one another.  LBM_ETIMEOUT
+ * when the first launch gave up, came back with its words clear, and the second
+ * one completed every item; LBM_OK otherwise; errors as above.  Synchronises
+ * `stream`; allocates and frees a few kilobytes. */
+int lbm_selftest_chain_timeout(long long cycles, void* stream);
+
 /* Measured FP64 fused multiply-add rate of the current device (no
  * counterpart in the paper): a kernel of independent DFMA chains on every SM,
  * timed with CUDA events after one warm-up launch; *flops_per_s receives

@@ -62,22 +62,28 @@ __device__ __forceinline__ int chain_item(const ChainTiles& ct, int item, int ns
 }
 
 // tile_fn(tile, parity, ready): advances one tile; calls ready() from every
-// thread before it reads any population.
+// thread before it reads any population.  limit: SM cycles after which a wait
+// gives up.
 template <int THREADS, typename TileFn>
 __device__ __forceinline__ void chain_run(const ChainTiles& ct, int nsteps, int parity0, int rot, uint32_t* err,
-                                          TileFn tile_fn) {
-    __shared__ int s_tile, s_step, s_stop, s_last;
+                                          TileFn tile_fn, long long limit = kWaitCycles) {
+    // s_stop: a wait of this item gave up.  Items alternate between its two
+    // words, so that no wait writes the word that the threads are still reading:
+    // all of them leave the loop at the same item, or none (tile_fn and ready
+    // hold barriers of the whole CTA).
+    __shared__ int s_tile, s_step, s_stop[2], s_last;
     const int t = threadIdx.x;
     if (t == 0) {
         int st = 0;
         s_tile = chain_item(ct, atomicAdd(&ct.ctl->next, 1), nsteps, rot, st);
         s_step = st;
-        s_stop = 0;
+        s_stop[0] = s_stop[1] = 0;
     }
     __syncthreads();
-    for (;;) {
+    bool stop = false;
+    for (int word = 0;; word ^= 1) {
         const int tile = s_tile, step = s_step;
-        if (tile < 0 || s_stop) break;
+        if (tile < 0 || stop) break;
         int ntile = -1, nstep = 0;
         tile_fn(tile, (parity0 + step) & 1, [&] {
             if (t < 32) {
@@ -85,10 +91,10 @@ __device__ __forceinline__ void chain_run(const ChainTiles& ct, int nsteps, int 
                 if (d >= 0 && ld_acquire(&ct.flags[d]) < step) {
                     const long long start = clock64();
                     while (ld_acquire(&ct.flags[d]) < step) {
-                        if (clock64() - start > kWaitCycles || ld_relaxed(&ct.ctl->abort)) {
+                        if (clock64() - start > limit || ld_relaxed(&ct.ctl->abort)) {
                             atomicOr(err, ERR_TIMEOUT);
                             atomicExch(&ct.ctl->abort, 1);
-                            s_stop = 1;
+                            s_stop[word] = 1;
                             break;
                         }
                     }
@@ -104,7 +110,8 @@ __device__ __forceinline__ void chain_run(const ChainTiles& ct, int nsteps, int 
             }
         });
         __syncthreads();
-        if (t == 0 && !s_stop) st_release(&ct.flags[tile], step + 1);
+        stop = s_stop[word] != 0;   // (written again two items on at the earliest)
+        if (t == 0 && !stop) st_release(&ct.flags[tile], step + 1);
     }
     // the last CTA leaves the control words and flags zero for the next launch
     if (t == 0) {

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "lbm.h"
+#include "lbm_chain.cuh"
 #include "lbm_kernels.cuh"
 
 namespace {
@@ -41,6 +42,87 @@ extern "C" int lbm_selftest_wait_timeout(long long cycles, void* stream) {
     cudaFree(d_err);
     if (e != cudaSuccess) return LBM_ECUDA;
     return (h_err & sc::ERR_TIMEOUT) ? LBM_ETIMEOUT : LBM_OK;
+}
+
+namespace {
+
+constexpr int kChainThreads = 128, kChainTilesTest = 64, kChainStepsTest = 6;
+
+// A chained launch whose tiles compute nothing but hold the barriers of the
+// bidirectional march; done[tile] counts the steps of each tile.
+__global__ void __launch_bounds__(kChainThreads) k_chain_selftest(sc::ChainTiles ct, int nsteps, long long limit,
+                                                                 uint32_t* err, int* done) {
+    __shared__ int s_sum[2];
+    sc::chain_run<kChainThreads>(
+        ct, nsteps, 0, 3, err,
+        [&](int tile, int, auto ready) {
+            const int t = threadIdx.x, group = t / 64;
+            ready();
+            for (int k = 0; k < 3; ++k) {
+                if (t % 64 == 0) s_sum[group] = tile;
+                if (k == 0) __syncthreads();
+                else sc::bar_group<64>(group);
+            }
+            if (t == 0) atomicAdd(&done[s_sum[0]], 1);
+        },
+        limit);
+}
+
+}  // namespace
+
+extern "C" int lbm_selftest_chain_timeout(long long cycles, void* stream) {
+    if (cycles < 1000 || cycles > 4000000000LL) return LBM_EINVAL;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    constexpr int N = kChainTilesTest;
+    // deps, span, control words, flags (one more that no tile sets), counts, error word
+    constexpr int kSpan = N * sc::kChainDeps, kCtl = kSpan + 2 * N, kFlags = kCtl + 4, kDone = kFlags + N + 1,
+                  kErr = kDone + N, kWords = kErr + 1;
+    int tab[kWords];
+    int* d = nullptr;
+    if (cudaMalloc(&d, sizeof(tab)) != cudaSuccess) {
+        cudaGetLastError();
+        return LBM_ENOMEM;
+    }
+    bool gave_up = false, clean = false, complete = true;
+    cudaError_t e = cudaSuccess;
+    for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
+        // first every tile waits for the flag that nothing sets; then, with the control
+        // words and flags that this launch left behind, for itself and its left neighbour
+        for (int i = 0; i < kSpan; ++i) tab[i] = -1;
+        for (int i = 0; i < N; ++i) {
+            int* dep = tab + i * sc::kChainDeps;
+            dep[i % sc::kChainDeps] = pass == 0 ? N : (i + N - 1) % N;
+            if (pass == 1) dep[(i + 1) % sc::kChainDeps] = i;
+            tab[kSpan + 2 * i] = 0;
+            tab[kSpan + 2 * i + 1] = N;
+        }
+        if (pass == 0)
+            for (int i = kCtl; i < kWords; ++i) tab[i] = 0;
+        e = cudaMemcpyAsync(d, tab, (pass == 0 ? kWords : kCtl) * sizeof(int), cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess && pass == 1) e = cudaMemsetAsync(d + kDone, 0, (N + 1) * sizeof(int), s);
+        if (e == cudaSuccess) {
+            const sc::ChainTiles ct{nullptr, reinterpret_cast<const int2*>(d + kSpan), d, d + kFlags,
+                                    reinterpret_cast<sc::ChainCtl*>(d + kCtl), N};
+            k_chain_selftest<<<24, kChainThreads, 0, s>>>(ct, kChainStepsTest, cycles,
+                                                          reinterpret_cast<uint32_t*>(d + kErr), d + kDone);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaMemcpyAsync(tab, d, sizeof(tab), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) break;
+        bool zero = true;
+        for (int i = kCtl; i < kDone; ++i) zero = zero && tab[i] == 0;
+        if (pass == 0) {
+            gave_up = (tab[kErr] & (int)sc::ERR_TIMEOUT) != 0;
+            clean = zero;
+        } else {
+            for (int i = 0; i < N; ++i) complete = complete && tab[kDone + i] == kChainStepsTest;
+            complete = complete && zero && tab[kErr] == 0;
+        }
+    }
+    cudaFree(d);
+    if (e != cudaSuccess) return LBM_ECUDA;
+    return gave_up && clean && complete ? LBM_ETIMEOUT : LBM_OK;
 }
 
 namespace {
