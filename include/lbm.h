@@ -377,7 +377,8 @@ int lbm_set_tiling(lbm_t* h, int tile_w, int tile_h);
  *                         nx, ny >= 4.
  * depth is read by LBM_KERNEL_ASYNC, LBM_KERNEL_TMA and LBM_KERNEL_RING and
  * must be 4 for the others.  lbm_set_schedule returns LBM_EINVAL for an unsupported
- * combination, leaving the schedule unchanged. */
+ * combination, and LBM_ENOMEM where the schedule's tables do not fit in memory;
+ * both leave the schedule unchanged. */
 #define LBM_KERNEL_REGISTER 0
 #define LBM_KERNEL_ASYNC 1
 #define LBM_KERNEL_TMA 2

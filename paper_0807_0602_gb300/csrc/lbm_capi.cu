@@ -415,6 +415,26 @@ int upload_tiles(lbm_t* h, int W, int R) {
     return LBM_OK;
 }
 
+struct Sched {
+    int W, R, kvar, depth;
+};
+
+// Changes the handle's schedule, or leaves it as it was and returns the error
+// (the new one's tables may not fit in memory): the old schedule's tables are
+// then written again, into the allocations that held them.
+int use_schedule(lbm_t* h, const Sched& s) {
+    const Sched old{h->tile_w, h->tile_h, h->kvar, h->depth};
+    h->kvar = s.kvar;
+    h->depth = s.depth;
+    const int rc = upload_tiles(h, s.W, s.R);
+    if (rc == LBM_OK) return rc;
+    h->kvar = old.kvar;
+    h->depth = old.depth;
+    const int back = upload_tiles(h, old.W, old.R);
+    if (back != LBM_OK && h->sticky == LBM_OK) h->sticky = back;   // no step may run on half a schedule
+    return rc;
+}
+
 sc::LogCtl logctl(lbm_t* h) {
     sc::LogCtl lc;
     lc.count = h->d_logcount;
@@ -701,10 +721,6 @@ int wave_height(lbm_t* h, int W, int waves) {
     return lo;
 }
 
-struct Sched {
-    int W, R, kvar, depth;
-};
-
 // The schedule of a handle that nobody has chosen one for, by the size of its
 // runs.  Measured on a GB300, us per step:
 //   - FP32 and FP16S up to 130 000 nodes: one node per thread (32 x 6 tiles) and
@@ -824,9 +840,7 @@ int autotune(lbm_t* h, int64_t* n) {
     // time candidate c over `steps` steps (after one untimed step); ms < 0 on error
     auto time_cand = [&](const Cand& c, int steps, float& ms) {
         ms = -1.f;
-        h->kvar = c.kvar;
-        h->depth = c.depth;
-        if ((rc = upload_tiles(h, c.W, c.R))) return;
+        if ((rc = use_schedule(h, c))) return;
         if ((rc = advance(h, 1))) return;
         cudaError_t e = cudaEventRecord(e0, h->stream);
         if (e == cudaSuccess && (rc = advance(h, steps))) return;
@@ -876,9 +890,7 @@ int autotune(lbm_t* h, int64_t* n) {
     cudaEventDestroy(e1);
     if (rc) return rc;
     h->tuned = true;
-    h->kvar = bw.kvar;
-    h->depth = bw.depth;
-    return upload_tiles(h, bw.W, bw.R);
+    return use_schedule(h, bw);
 }
 
 int check_run(const lbm_t* h, int run) {
@@ -1356,15 +1368,15 @@ int lbm_get_tiling(const lbm_t* h, int* tile_w, int* tile_h) {
 
 int lbm_set_tiling(lbm_t* h, int tile_w, int tile_h) {
     if (!h) return LBM_EINVAL;
-    if (!schedule_ok(h, tile_w, tile_h, h->kvar, h->depth)) {
+    Sched s{tile_w, tile_h, h->kvar, h->depth};
+    if (!schedule_ok(h, tile_w, tile_h, s.kvar, s.depth)) {
         // the current kernel does not take this tiling: a march does
-        const int march = schedule_ok(h, tile_w, tile_h, 6, 4) ? 6 : 0;
-        if (!schedule_ok(h, tile_w, tile_h, march, 4)) return LBM_EINVAL;
-        h->kvar = march;
-        h->depth = 4;
+        s.kvar = schedule_ok(h, tile_w, tile_h, 6, 4) ? 6 : 0;
+        s.depth = 4;
+        if (!schedule_ok(h, tile_w, tile_h, s.kvar, s.depth)) return LBM_EINVAL;
     }
     h->tuned = true;
-    return upload_tiles(h, tile_w, tile_h);
+    return use_schedule(h, s);
 }
 
 int lbm_get_schedule(const lbm_t* h, int* tile_w, int* tile_h, int* kernel, int* depth) {
@@ -1396,9 +1408,7 @@ int lbm_set_schedule(lbm_t* h, int tile_w, int tile_h, int kernel, int depth) {
         if (rc) return rc;
     }
     h->tuned = true;
-    h->kvar = kernel;
-    h->depth = depth;
-    return upload_tiles(h, tile_w, tile_h);
+    return use_schedule(h, {tile_w, tile_h, kernel, depth});
 }
 
 namespace {

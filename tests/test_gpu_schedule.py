@@ -1,0 +1,53 @@
+"""Changing a handle's schedule: what happens when memory runs out."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(nx, ny):
+    geom = W.capillary_geometry(nx, ny, nx // 8, nx - nx // 8, 0, ny - 3)
+    nA, nB = W.random_fields(geom, 5, 0.2, 1.2)
+    return dict(geom=geom, params=W.params(0.9, 1.0, 0.9, -0.1, 0.05), init=("fields", nA, nB))
+
+
+# (precision, grid, schedule before, schedules whose tables need memory beyond
+# the starting schedule's: kernel 9 with two rows, kernel 8)
+@pytest.mark.parametrize("prec,grid,before,wanted", [
+    ("f64", (300, 60), (64, 16, 9, 4), [(64, 16, 12, 4), (64, 1, 9, 4), (64, 1, 12, 4)]),
+    ("f64", (300, 60), (64, 16, 12, 4), [(64, 1, 12, 4), (64, 1, 9, 4), (128, 1, 6, 4)]),
+    ("f32", (700, 200), (128, 16, 6, 4), [(32, 6, 13, 4), (128, 4, 10, 4), (64, 1, 9, 4)]),
+])
+def test_a_schedule_that_does_not_fit_in_memory_leaves_the_old_one(monkeypatch, prec, grid, before, wanted):
+    """The old schedule stays and works (kernels 12 and 13 used to be selected
+    without their tables, which the next step would have read)."""
+    from paper_0807_0602_gb300 import _lib as L
+    from paper_0807_0602_gb300 import lbm
+    from paper_0807_0602_gb300.build import build
+    build()
+    deny = []
+
+    class Denying(lbm._TorchAllocator):
+        def _alloc(self, ctx, nbytes, stream):
+            return None if deny else super()._alloc(ctx, nbytes, stream)
+
+    monkeypatch.setattr(lbm, "_TorchAllocator", Denying)
+    run = _run(*grid)
+    with lbm.Lattice(run, precision=prec, tile=before[:2], kernel=before[2:]) as a, \
+            lbm.Lattice(run, precision=prec, tile=(128, 4), kernel=(6, 4)) as b:
+        a.step(3)
+        for s in wanted:
+            deny.append(1)
+            with pytest.raises(L.LbmError) as e:
+                a.schedule = s
+            assert e.value.code == L.LBM_ENOMEM
+            deny.clear()
+            assert a.schedule == before and a.status() == L.LBM_OK
+            a.step(6)
+        a.schedule = wanted[0]
+        a.step(5)
+        b.step(3 + 6 * len(wanted) + 5)
+        assert a.schedule == wanted[0]
+        assert np.array_equal(a.populations(), b.populations())
