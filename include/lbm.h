@@ -117,7 +117,9 @@ typedef struct lbm_geometry {
 } lbm_geometry;
 
 /* Device allocator supplied by the caller (for instance a framework's
- * caching allocator).  alloc returns NULL on failure. */
+ * caching allocator).  alloc returns NULL on failure; memory that does not
+ * start on a 16-byte boundary is given back and asked for again, 16 bytes
+ * larger.  free gets the pointers and sizes of alloc. */
 typedef void* (*lbm_alloc_fn)(void* ctx, size_t bytes, void* stream);
 typedef void (*lbm_free_fn)(void* ctx, void* ptr, size_t bytes, void* stream);
 

@@ -125,8 +125,17 @@ void* dalloc(lbm_t* h, size_t bytes) {
         cudaGetLastError();
         p = nullptr;
     }
-    if (p) h->allocs.push_back({p, bytes});
-    return p;
+    // bulk copies and 16-byte accesses rely on that alignment, which a caller's
+    // allocator need not give: ask it once more for room to round up
+    const uintptr_t unit = 16;
+    if (p && reinterpret_cast<uintptr_t>(p) % unit != 0) {
+        h->opt.free(h->opt.alloc_ctx, p, bytes, h->stream);
+        bytes += unit;
+        p = h->opt.alloc(h->opt.alloc_ctx, bytes, h->stream);
+    }
+    if (!p) return nullptr;
+    h->allocs.push_back({p, bytes});   // as the allocator gave it
+    return reinterpret_cast<void*>((reinterpret_cast<uintptr_t>(p) + unit - 1) / unit * unit);
 }
 
 void dfree_all(lbm_t* h) {

@@ -99,3 +99,39 @@ def test_log_records_equal_the_separate_readouts(prec):
                     assert np.array_equal(rec[1:4], lat.interface(r))
                 else:
                     assert np.all(np.isnan(rec[1:4]))
+
+
+@pytest.mark.parametrize("prec", ["f32", "f16s", "f64"])
+@pytest.mark.parametrize("kernel", [None, (128, 4, 2, 4), (64, 8, 7, 4)])
+def test_memory_off_16_bytes(monkeypatch, prec, kernel):
+    """A caller's allocator may return memory on 8-byte boundaries only; column
+    windows and the bulk-copy kernels read 16 bytes at a time."""
+    from paper_0807_0602_gb300 import lbm
+    from paper_0807_0602_gb300.build import build
+    build()
+    given, wrong, off = {}, [], 8
+
+    class Off8(lbm._TorchAllocator):
+        def _alloc(self, ctx, nbytes, stream):
+            p = super()._alloc(ctx, nbytes + off, stream)
+            if p is not None:
+                given[p + off] = nbytes
+                return p + off
+
+        def _free(self, ctx, ptr, nbytes, stream):
+            if given.pop(int(ptr), None) != nbytes:
+                wrong.append((ptr, nbytes))
+            super()._free(ctx, int(ptr) - off, nbytes + off, stream)
+
+    with _box(64, 24, prec) as lat:
+        lat.step(5)
+        want = lat.populations()
+    monkeypatch.setattr(lbm, "_TorchAllocator", Off8)
+    kw = {} if kernel is None else dict(tile=kernel[:2], kernel=kernel[2:])
+    with _box(64, 24, prec, **kw) as lat:
+        info = lat.run_info()
+        assert (info.base[0] | info.base[1]) % 16 == 0
+        lat.step(5)
+        assert np.array_equal(lat.get_columns(0, 64).cpu().numpy(), want)
+        assert np.array_equal(lat.get_columns(8, 16).cpu().numpy(), want[..., 8:24])
+    assert not given and not wrong   # every allocation given back as it was
