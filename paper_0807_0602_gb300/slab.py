@@ -109,14 +109,14 @@ def exchange_local(slabs) -> None:
 def _step_native(slabs, n: int) -> bool:
     """The steps and exchanges of GPU slabs of one stream and device by one
     library call (one copy kernel per step); False if these slabs need the
-    general exchange."""
+    general exchange (the library takes slabs of four owned columns and more)."""
     from . import lbm as B
     if not 1 <= len(slabs) <= 32 or any(type(s) is not Slab or type(s.lat) is not B.Lattice for s in slabs):
         return False
     lats = [s.lat for s in slabs]
     one = lats[0]
     if len({id(a) for a in lats}) != len(lats) or any(
-            not a._h or a.nruns != 1 or a.precision != one.precision or a.device != one.device
+            not a._h or a.nruns != 1 or a.shapes[0][1] < 8 or a.precision != one.precision or a.device != one.device
             or a.stream.cuda_stream != one.stream.cuda_stream or a.shapes[0][0] != one.shapes[0][0] for a in lats):
         return False
     handles = (ctypes.c_void_p * len(lats))(*[a._h.value for a in lats])

@@ -59,3 +59,22 @@ def test_other_slabs_take_the_general_exchange():
     SL.step_local(a, 5)
     _general(b, 5)
     assert np.array_equal(_all(a), _all(b))
+
+
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+@pytest.mark.parametrize("cuts", [(0, 2, 40), (0, 3, 5, 40), (0, 37, 40)])
+def test_slabs_of_two_or_three_columns_step(prec, cuts):
+    """Slabs built by hand may be narrower than the library's call takes: they
+    go through the general exchange and still equal the undivided run."""
+    from paper_0807_0602_gb300 import slab as SL
+    from paper_0807_0602_gb300.lbm import Lattice
+    geom = W.capillary_geometry(40, 12, 5, 37, 0, 11)
+    nA, nB = W.random_fields(geom, 4, 0.2, 1.2)
+    run = dict(geom=geom, params=W.params(1.2, 1.0, 0.9, -0.1, 0.05), init=("fields", nA, nB))
+    _slabs(40, 12, 1)   # (builds the library)
+    slabs = [SL.Slab(run, a, b, nA, nB, precision=prec) for a, b in zip(cuts, cuts[1:])]
+    with Lattice(run, precision=prec) as whole:
+        SL.step_local(slabs, 7)
+        whole.step(7)
+        got = np.concatenate([s.owned(s.lat.populations()) for s in slabs], axis=-1)
+        assert np.array_equal(got, whole.populations())
