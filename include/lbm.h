@@ -145,7 +145,9 @@ typedef void (*lbm_free_fn)(void* ctx, void* ptr, size_t bytes, void* stream);
  *               lbm_get_schedule reports them; autotune, lbm_set_tiling or
  *               lbm_set_schedule change them.  Results do not depend on it.
  * graph_chunk   steps captured per CUDA graph when the log is off (0 = 64;
- *               -1 = launch every step directly).
+ *               -1 = no graphs: launch every step directly).
+ *               LBM_KERNEL_CHAIN, which FP64 handles may start with, takes
+ *               several steps per launch in either case.
  * rho_ref       FP16S shift per species (ignored otherwise).
  * rho_bulk      base of the precursor threshold rho_bulk / 3 (0 = 2.0).
  * body          constant body force per particle, added to F_k / n_k of
@@ -369,9 +371,12 @@ int lbm_set_tiling(lbm_t* h, int tile_w, int tile_h);
  *                         CTAs draw (step, tile) items from a device counter
  *                         and wait for the neighbouring tiles' step before
  *                         only (LBM_F64; tile_w 64).  lbm_step then issues
- *                         all its steps up to the next log record as one
- *                         launch (graph_chunk > 0: that many), inside a CUDA
- *                         graph where the log is on and whole.
+ *                         its steps up to the next log record (graph_chunk >
+ *                         0 and the log off: up to that many) in launches of
+ *                         some 10 ms, 8 steps at least (with graph_chunk = -1
+ *                         too), inside a CUDA graph where the log is on and
+ *                         the interval whole.  Choose LBM_KERNEL_BIDIR for
+ *                         one launch per step.
  *   LBM_KERNEL_TWO_STEP   LBM_KERNEL_TILE with tile_w 32 and tile_h 6, but four
  *                         steps at a time are two launches of two steps each
  *                         (the last step of an lbm_step call or a log interval

@@ -453,12 +453,14 @@ sc::LogCtl logctl(lbm_t* h) {
 }
 
 // Issues n chained steps on stream s (parity = t & 1 of the first), as many to
-// a launch as its item numbers allow.
+// a launch as chain_launch_steps allows.
 cudaError_t issue_chain(lbm_t* h, int parity, int64_t n, cudaStream_t s) {
     const sc::ChainTiles ct = chain_tables(h);
+    int64_t nodes = 0;
+    for (const RunDesc& rd : h->runs) nodes += rd.nodes;
     cudaError_t e = cudaSuccess;
     while (n > 0 && e == cudaSuccess) {
-        const int m = (int)sc::chain_launch_steps(n, ct.ntiles);
+        const int m = (int)sc::chain_launch_steps(n, ct.ntiles, nodes);
         // a single step has nothing to chain: the bidirectional march takes the same tiles
         if (m == 1)
             e = dispatch_step(h, [&](auto L) {

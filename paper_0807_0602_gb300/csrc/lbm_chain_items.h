@@ -15,9 +15,21 @@ namespace sc {
 // one number beyond the last item.
 constexpr long long kChainItems = 1LL << 30;
 
-// Steps of the next chained launch of n steps (n >= 1) over ntiles tiles.
-LBM_HD_ITEMS long long chain_launch_steps(long long n, long long ntiles) {
-    const long long most = ntiles < kChainItems ? kChainItems / (ntiles > 0 ? ntiles : 1) : 1;
+// A launch keeps most of every SM's shared memory from other streams' work until
+// it ends, so its length is bounded, too: 2^25 nodes times steps are 13 ms on a
+// GB300 (2048 x 130: 126 steps; 30 000 nodes, where steps are longer than their
+// nodes ask for: 1100 steps, some 22 ms).  Between launches the tiles drain,
+// about a wave of them, below a hundredth of that.  Never less than 8 steps: on
+// larger grids a single step takes milliseconds.
+constexpr long long kChainNodeSteps = 1LL << 25, kChainMinSteps = 8;
+
+// Steps of the next chained launch of n steps (n >= 1) over ntiles tiles of
+// `nodes` nodes in all.
+LBM_HD_ITEMS long long chain_launch_steps(long long n, long long ntiles, long long nodes) {
+    const long long items = ntiles < kChainItems ? kChainItems / (ntiles > 0 ? ntiles : 1) : 1;
+    const long long work = nodes > 0 ? kChainNodeSteps / nodes : n;
+    long long most = work > kChainMinSteps ? work : kChainMinSteps;
+    if (most > items) most = items;
     return n < most ? n : most;
 }
 

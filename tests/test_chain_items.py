@@ -25,10 +25,10 @@ int main() {
             // the first launches and the last one (all between are alike)
             long long left = n;
             for (int k = 0; k < 4 && left > 0; ++k) {
-                const long long m = chain_launch_steps(left, nt);
+                const long long m = chain_launch_steps(left, nt, 1);
                 ++launches;
                 bad += m < 1 || m > left || (m > 1 && m * nt + ctas > INT_MAX);
-                bad += m < left && (m + 1) * nt <= kChainItems;   // no shorter than need be
+                bad += m < left && (m + 1) * nt <= kChainItems && m + 1 <= kChainNodeSteps;   // no shorter than need be
                 if (m > 1 && m * nt + ctas <= INT_MAX) {
                     // the tiles of the highest and of the drawn-beyond numbers, in runs of `per` tiles
                     for (long long per : {nt, (nt + 2) / 3})
@@ -44,6 +44,14 @@ int main() {
                 }
                 left -= m;
             }
+        }
+    // the length of a launch: 2^25 nodes times steps, or 8 steps of a larger grid
+    for (long long nodes : {1LL, 30000LL, 266240LL, 1310720LL, 5000000LL, 67108864LL, 1LL << 30})
+        for (long long n : {1LL, 7LL, 8LL, 25LL, 50LL, 1000LL, 100000000LL}) {
+            const long long nt = nodes / 62 + 1, m = chain_launch_steps(n, nt, nodes);
+            bad += m < 1 || m > n || (m > 8 && m * nodes > (1LL << 25));
+            bad += m < n && m < 8 && nt * 8 <= kChainItems;
+            bad += n * nodes <= (1LL << 25) && n * nt <= kChainItems && m != n;
         }
     // every tile of every step once
     for (int nt : {1, 2, 7, 40})

@@ -155,3 +155,22 @@ def test_two_step_tilings_are_validated():
     with Lattice(_run(64, 3, "box"), precision="f32") as lat:   # fewer than four rows
         with pytest.raises(L.LbmError):
             lat.schedule = (32, 6, 13, 4)
+
+
+@pytest.mark.parametrize("chunk", [0, -1, 70])
+def test_steps_of_several_chained_launches(chunk):
+    """800 000 nodes: at most 41 steps to a launch, within the log's graph, too."""
+    run = dict(_run(2000, 400, "cap"), params=W.params(1.0, 1.0, 1.0, -0.2), init=("slab", 0, 700))
+    for every in (0, 100):
+        kw = dict(precision="f64", graph_chunk=chunk, log_every=every, log_capacity=8 if every else 0)
+        with Lattice(run, tile=(64, 16), kernel=(CHAIN, 4), **kw) as a, Lattice(run, tile=(64, 16), kernel=(9, 4), **kw) as b:
+            for n in (1, 130, 269):
+                a.step(n)
+                b.step(n)
+                assert a.status() == 0 and a.t == b.t
+            for p, q in zip(a.densities(), b.densities()):
+                assert np.array_equal(p, q)
+            for p, q in zip(a.velocity(), b.velocity()):   # reads the state of the step before
+                assert np.array_equal(p, q)
+            if every:
+                assert np.array_equal(a.log(), b.log())
