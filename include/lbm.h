@@ -136,7 +136,8 @@ typedef void (*lbm_free_fn)(void* ctx, void* ptr, size_t bytes, void* stream);
  *               tiles fill one or two waves of resident CTAs, and for a
  *               handle of one run LBM_KERNEL_BIDIR_JIT at those heights
  *               (compiled once per grid and strip width, about 0.5 s each,
- *               where NVRTC is available; left out otherwise).  These are
+ *               where NVRTC is available; left out otherwise), and the
+ *               schedule that the handle has.  These are
  *               real steps: tilings change only the schedule, and results
  *               are bit-identical for every tiling.
  * tile_w        a hint (64, 128 or 256; 0 = default 128), and

@@ -1,4 +1,5 @@
-"""Changing a handle's schedule: what happens when memory runs out."""
+"""Changing a handle's schedule: what happens when memory runs out, and that
+the autotuner can stay with the schedule it starts from."""
 import numpy as np
 import pytest
 
@@ -50,4 +51,22 @@ def test_a_schedule_that_does_not_fit_in_memory_leaves_the_old_one(monkeypatch, 
         a.step(5)
         b.step(3 + 6 * len(wanted) + 5)
         assert a.schedule == wanted[0]
+        assert np.array_equal(a.populations(), b.populations())
+
+
+def test_the_autotuner_times_the_starting_schedule():
+    """1024 x 66 FP32 starts with two steps per launch (3.0 us per step), a
+    quarter faster than every other kernel: it has to be among the finalists."""
+    from paper_0807_0602_gb300 import lbm
+    from paper_0807_0602_gb300.build import build
+    build()
+    run = _run(1024, 66)
+    run.update(params=W.params(1.0, 1.0, 1.0, -0.2), init=("slab", 0, 400))
+    with lbm.Lattice(run, precision="f32", autotune=True) as a, lbm.Lattice(run, precision="f32") as b:
+        start = a.schedule
+        assert start == (32, 6, 13, 4) and start == b.schedule
+        a.step(3000)
+        b.step(3000)
+        assert start in [s for s, _ in a.tuning()]
+        assert a.schedule == min(a.tuning(), key=lambda c: c[1])[0]
         assert np.array_equal(a.populations(), b.populations())
