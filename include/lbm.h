@@ -417,7 +417,9 @@ int lbm_set_schedule(lbm_t* h, int tile_w, int tile_h, int kernel, int depth);
  * path; lbm_load re-creates the handle so that stepping on gives results
  * bit-identical to an uninterrupted run.  Both synchronise.  LBM_EIO on
  * file errors.  The file keeps alpha and molecular_mass (format version 2);
- * version 1 files load with the defaults 4/9 and 1. */
+ * version 1 files load with the defaults 4/9 and 1.  It also keeps the
+ * schedule where lbm_set_tiling, lbm_set_schedule or the autotuner chose it;
+ * otherwise the library chooses one on load. */
 int lbm_save(lbm_t* h, const char* path);
 int lbm_load(const char* path, const lbm_options* opt, lbm_t** out);
 

@@ -91,6 +91,7 @@ struct lbm_s {
     std::vector<Alloc> allocs;
     std::map<GraphKey, cudaGraphExec_t> graphs;
     bool tuned = false;
+    bool chosen = false;           // the schedule was set by the caller or found by the autotuner
     std::vector<int> tune_sched;   // the tuner's finalists, 4 ints each (tile_w, tile_h, kernel, depth)
     std::vector<float> tune_ms;    // and their best ms per step over the final rounds
     int sticky = LBM_OK;
@@ -436,7 +437,10 @@ int use_schedule(lbm_t* h, const Sched& s) {
     h->kvar = s.kvar;
     h->depth = s.depth;
     const int rc = upload_tiles(h, s.W, s.R);
-    if (rc == LBM_OK) return rc;
+    if (rc == LBM_OK) {
+        h->chosen = true;
+        return rc;
+    }
     h->kvar = old.kvar;
     h->depth = old.depth;
     const int back = upload_tiles(h, old.W, old.R);
@@ -1437,7 +1441,8 @@ const char kMagic[8] = {'S', 'C', 'L', 'B', 'M', 'C', 'K', '1'};
 
 struct CkHeader {
     char magic[8];
-    int32_t version, precision, nruns, log_every, log_capacity, tile_w, tile_h, reserved;
+    int32_t version, precision, nruns, log_every, log_capacity, tile_w, tile_h;
+    uint32_t sched;   // a chosen schedule (pack_sched), or 0: the library chooses on load
     int64_t t, nlog;
     double rho_ref[2], rho_bulk, body[2];
 };
@@ -1445,6 +1450,14 @@ struct CkHeader {
 struct CkModel {
     double alpha[2], molecular_mass[2];
 };
+// kernel + 1, depth, tile_w / 32 (4 bits each) and tile_h; 0 for what does not fit
+uint32_t pack_sched(const Sched& s) {
+    if (s.W % 32 || s.W / 32 > 15 || s.depth > 15 || s.kvar > 14 || s.R >= (1 << 20)) return 0;
+    return (uint32_t)(s.kvar + 1) | (uint32_t)s.depth << 4 | (uint32_t)(s.W / 32) << 8 | (uint32_t)s.R << 12;
+}
+Sched unpack_sched(uint32_t v) {
+    return {(int)(v >> 8 & 15) * 32, (int)(v >> 12), (int)(v & 15) - 1, (int)(v >> 4 & 15)};
+}
 struct CkRun {
     int32_t nx, ny, cap_x0, cap_x1, y_bot, y_top, has_mask, reserved;
     double G, GwA, GwB, tauA, tauB;
@@ -1464,8 +1477,9 @@ int lbm_save(lbm_t* h, const char* path) {
     hd.nruns = h->nruns;
     hd.log_every = h->opt.log_every;
     hd.log_capacity = h->opt.log_capacity;
-    hd.tile_w = h->opt.tile_w;   // the options' values: schedules are chosen anew on load
+    hd.tile_w = h->opt.tile_w;
     hd.tile_h = h->opt.tile_h;
+    hd.sched = h->chosen ? pack_sched({h->tile_w, h->tile_h, h->kvar, h->depth}) : 0;
     hd.t = h->t;
     hd.nlog = h->nlog;
     hd.rho_ref[0] = h->opt.rho_ref[0];
@@ -1617,6 +1631,17 @@ int lbm_load(const char* path, const lbm_options* opt_in, lbm_t** out) {
     if (cudaMemcpy(h->d_logcount, &cnt, sizeof(cnt), cudaMemcpyHostToDevice) != cudaSuccess) {
         lbm_destroy(h);
         return LBM_ECUDA;
+    }
+    if (hd.sched) {
+        // the schedule changes no result: where it cannot be had (a kernel that needs
+        // the run-time compiler, memory) the handle keeps the one it starts with
+        const Sched sd = unpack_sched(hd.sched);
+        if (schedule_ok(h, sd.W, sd.R, sd.kvar, sd.depth)) use_schedule(h, sd);
+        if (h->sticky) {
+            rc = h->sticky;
+            lbm_destroy(h);
+            return rc;
+        }
     }
     *out = h;
     return LBM_OK;

@@ -1,5 +1,6 @@
-"""Changing a handle's schedule: what happens when memory runs out, and that
-the autotuner can stay with the schedule it starts from."""
+"""Changing a handle's schedule: what happens when memory runs out, that
+the autotuner can stay with the schedule it starts from, and that checkpoints
+keep a schedule somebody chose."""
 import numpy as np
 import pytest
 
@@ -70,3 +71,37 @@ def test_the_autotuner_times_the_starting_schedule():
         assert start in [s for s, _ in a.tuning()]
         assert a.schedule == min(a.tuning(), key=lambda c: c[1])[0]
         assert np.array_equal(a.populations(), b.populations())
+
+
+@pytest.mark.parametrize("prec,schedule", [
+    ("f32", (64, 5, 9, 4)), ("f32", (32, 14, 8, 4)), ("f32", (128, 4, 10, 3)), ("f16s", (256, 7, 2, 6)),
+    ("f64", (64, 3, 12, 4)), ("f64", (256, 100000, 0, 4)), ("f32", (64, 6, 11, 4)), ("f32", None), ("f64", None)])
+def test_checkpoints_keep_a_chosen_schedule(tmp_path, prec, schedule):
+    from paper_0807_0602_gb300 import lbm
+    from paper_0807_0602_gb300.build import build
+    build()
+    path = str(tmp_path / "state")
+    with lbm.Lattice(_run(300, 40), precision=prec) as a:
+        first = a.schedule
+        if schedule is not None:
+            a.schedule = schedule
+        a.step(9)
+        a.save(path)
+        a.step(8)
+        with lbm.Lattice.load(path) as b:
+            assert b.schedule == (schedule or first)
+            b.step(8)
+            assert np.array_equal(a.populations().view(np.uint8), b.populations().view(np.uint8))
+
+
+def test_checkpoints_keep_a_chosen_tiling(tmp_path):
+    from paper_0807_0602_gb300 import lbm
+    from paper_0807_0602_gb300.build import build
+    build()
+    path = str(tmp_path / "state")
+    with lbm.Lattice(_run(300, 40), precision="f32") as a:
+        a.tiling = (128, 16)
+        a.step(9)
+        a.save(path)
+        with lbm.Lattice.load(path) as b:
+            assert b.tiling == (128, 16) and b.schedule == a.schedule
