@@ -140,11 +140,12 @@ typedef void (*lbm_free_fn)(void* ctx, void* ptr, size_t bytes, void* stream);
  *               schedule that the handle has.  These are
  *               real steps: tilings change only the schedule, and results
  *               are bit-identical for every tiling.
- * tile_w        a hint (64, 128 or 256; 0 = default 128), and
- * tile_h        another (0 = default 4): the library chooses the step kernel
- *               and its tiling from the precision and the runs' sizes, and
- *               lbm_get_schedule reports them; autotune, lbm_set_tiling or
- *               lbm_set_schedule change them.  Results do not depend on it.
+ * tile_w        0, 64, 128 or 256, and
+ * tile_h        0 or more: checked, kept in checkpoints and not used.  A handle
+ *               starts with a step kernel and tiling that the library chooses
+ *               from the precision and the runs' sizes (lbm_get_schedule
+ *               reports them); lbm_set_tiling, lbm_set_schedule or autotune
+ *               change them.  Results do not depend on them.
  * graph_chunk   steps captured per CUDA graph when the log is off (0 = 64;
  *               -1 = no graphs: launch every step directly).
  *               LBM_KERNEL_CHAIN, which FP64 handles may start with, takes
@@ -208,7 +209,7 @@ typedef struct lbm_run_info {
     void* base[2];
 } lbm_run_info;
 
-/* Fills opt with the defaults documented above (FP32, no log, hint 128x4,
+/* Fills opt with the defaults documented above (FP32, no log, tile 128x4,
  * alpha 4/9, molecular mass 1). */
 void lbm_default_options(lbm_options* opt);
 

@@ -34,7 +34,7 @@ def measure_angles(couplings, G, tau_A=1.0, tau_B=1.0, steps=8000, precision="f3
     (G_Aw, G_Bw) pair, advanced together in one batched handle."""
     runs = [droplet_run(a, b, G, tau_A, tau_B, nx, ny, radius) for a, b in couplings]
     out = np.full(len(runs), np.nan)
-    with Lattice(runs, precision=precision, tile=(128, 16)) as lat:
+    with Lattice(runs, precision=precision) as lat:
         lat.step(steps)
         for i in range(len(runs)):
             nA, nB = lat.densities(i)
@@ -51,7 +51,7 @@ def angle_table(G_values, tau_B_values, couplings, tau_A=1.0, steps=8000, precis
     G_values, tau_B_values, couplings = (np.asarray(v, float) for v in (G_values, tau_B_values, couplings))
     runs = [droplet_run(a, 0.0, G, tau_A, tB) for G in G_values for tB in tau_B_values for a in couplings]
     out = np.full(len(runs), np.nan)
-    with Lattice(runs, precision=precision, tile=(128, 16)) as lat:
+    with Lattice(runs, precision=precision) as lat:
         lat.step(steps)
         for i in range(len(runs)):
             nA, nB = lat.densities(i)
@@ -111,7 +111,7 @@ def capillary_prefactors(samples, L_cap=256, steps=20000, log_every=100, precisi
     runs = [capillary_run(L_cap, int(s[5]), s[2], s[3], s[4], s[0], s[1]) for s in samples]
     kw = np.full(len(runs), np.nan)
     ap = np.full(len(runs), np.nan)
-    with Lattice(runs, precision=precision, tile=(128, 16), log_every=log_every,
+    with Lattice(runs, precision=precision, log_every=log_every,
                  log_capacity=steps // log_every + 2) as lat:
         lat.step(steps)
         for i, s in enumerate(samples):

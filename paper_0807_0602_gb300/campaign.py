@@ -109,7 +109,7 @@ def run(seed=4, n_train=1024, droplet_steps=20000, cap_train_steps=50000, n_targ
                              both=(-0.5, (0.0, 0.6)))
     ang = np.full(n_train, np.nan)
     runs = [Cb.droplet_run(X[i, 0], X[i, 1], X[i, 2], 1.0, 1.0, **DROP) for i in range(n_train)]
-    with Lattice(runs, precision="f32", tile=(128, 16)) as lat:
+    with Lattice(runs, precision="f32") as lat:
         lat.step(droplet_steps)
         for i in range(n_train):
             nA, nB = lat.densities(i)
@@ -164,7 +164,7 @@ def run(seed=4, n_train=1024, droplet_steps=20000, cap_train_steps=50000, n_targ
     # 5. verification: capillaries (FP32) and droplets (FP64)
     t0 = time.perf_counter()
     caps = [Cb.capillary_run(L_cap, H, 1.0, 1.0, 1.0, a, b) for a, b in prop]
-    with Lattice(caps, precision="f32", tile=(128, 16), log_every=500, log_capacity=cap_steps // 500 + 2) as lat:
+    with Lattice(caps, precision="f32", log_every=500, log_capacity=cap_steps // 500 + 2) as lat:
         lat.step(cap_steps)
         logs = [lat.log(i) for i in range(n_targets)]
     mu = 2.04 * 0.5 / 3.0

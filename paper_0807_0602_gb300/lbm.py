@@ -92,6 +92,11 @@ class Lattice:
     tau_A, tau_B; optional body, rho_bulk, alpha = (alpha_A, alpha_B) of
     Eqs. 3-5 and mass = (m_A, m_B), shared by all runs) and ``init`` (("slab", x_lo, x_hi),
     ("droplet", cx, cy, r) or ("fields", nA, nB)).
+
+    The library chooses the step kernel and its tiling; ``kernel = (kernel,
+    depth)`` together with ``tile = (tile_w, tile_h)`` sets both (see
+    ``schedule``).  ``tile`` without ``kernel`` is checked and not used; assign
+    ``tiling`` to change the tiling alone.
     """
 
     def __init__(self, runs, precision: str = "f32", log_every: int = 0, log_capacity: int = 0,

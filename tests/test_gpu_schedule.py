@@ -105,3 +105,44 @@ def test_checkpoints_keep_a_chosen_tiling(tmp_path):
         a.save(path)
         with lbm.Lattice.load(path) as b:
             assert b.tiling == (128, 16) and b.schedule == a.schedule
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32", "f16s"])
+def test_tilings_of_the_marches_equal_each_other(prec):
+    """Tiles of one row up to more rows than the run has, strips of each width,
+    with and without graphs.  (A tile given at creation without a kernel changes
+    nothing: the library chooses the schedule.)"""
+    from paper_0807_0602_gb300 import lbm
+    from paper_0807_0602_gb300.build import build
+    build()
+    geom = W.capillary_geometry(333, 37, 50, 300, 2, 30)
+    run = dict(geom=geom, params=W.params(1.2, 1.0, 0.9, -0.1, 0.05), init=("slab", 0, 120))
+    kw = dict(precision=prec, rho_ref=(1.0, 1.0))
+    with lbm.Lattice(run, **kw) as lat, lbm.Lattice(run, tile=(64, 3), **kw) as given:
+        assert lat.schedule == given.schedule
+        lat.step(23)
+        want = lat.populations().view(np.uint8)
+    for tile, chunk in (((128, 16), 0), ((64, 1), -1), ((64, 3), 5), ((256, 37), 0), ((128, 100), 7)):
+        kernels = {6, 0} if prec != "f64" or tile[0] < 256 else {0}
+        for kernel in kernels:
+            with lbm.Lattice(run, graph_chunk=chunk, tile=tile, kernel=(kernel, 4), **kw) as lat:
+                assert lat.schedule == (*tile, kernel, 4)
+                lat.step(23)
+                assert np.array_equal(lat.populations().view(np.uint8), want)
+
+
+def test_batched_runs_of_the_marches_equal_solo_runs():
+    from paper_0807_0602_gb300 import lbm
+    from paper_0807_0602_gb300.build import build
+    build()
+    runs = [W.capillary_run(L, H, 1.0 + 0.05 * j, 1.0, 0.8 + 0.1 * j, -0.1 * j)
+            for j, (L, H) in enumerate(((40, 6), (100, 13), (65, 30), (7, 3)))]
+    for kernel in (6, 0):
+        with lbm.Lattice(runs, precision="f32", tile=(64, 8), kernel=(kernel, 4)) as bat:
+            bat.step(40)
+            for r, run in enumerate(runs):
+                with lbm.Lattice(run, precision="f32", tile=(128, 16), kernel=(kernel, 4)) as solo:
+                    solo.step(40)
+                    assert np.array_equal(solo.populations(), bat.populations(r))
+                    assert np.array_equal(solo.interface(), bat.interface(r))
+                    assert np.array_equal(solo.mass(), bat.mass(r))
