@@ -140,7 +140,17 @@ class Network:
 
     def train_steps(self, x, t, idx, lr: float):
         """One training step per row of ``idx`` ([steps, n] row numbers of x
-        and t, the minibatches); returns the losses [steps]."""
+        and t, the minibatches); returns the losses [steps].  IndexError for a
+        row number outside x (the check waits for a CUDA idx)."""
+        idx = self._torch.as_tensor(idx).to(dtype=self._torch.int64)
+        if idx.numel():
+            lo, hi = (int(v) for v in idx.aminmax())
+            if lo < 0 or hi >= len(x):
+                raise IndexError(f"row numbers {lo} .. {hi} outside 0 .. {len(x) - 1}")
+        return self._train_steps(x, t, idx, lr)
+
+    def _train_steps(self, x, t, idx, lr: float):
+        """train_steps with row numbers known to be in range."""
         x, t = self._dev(x, N_IN), self._dev(t, N_OUT)
         idx = self._torch.as_tensor(idx).to(device="cuda", dtype=self._torch.int64).contiguous()
         assert idx.dim() == 2 and x.shape[0] == t.shape[0]
@@ -186,7 +196,7 @@ class Surrogate:
         # trains on this one's
         for s in range(0, steps, 64):
             idx = np.stack([rng.choice(n, size=min(batch, n), replace=False) for _ in range(min(64, steps - s))])
-            losses.append(self.net.train_steps(Xd, Td, idx, lr))
+            losses.append(self.net._train_steps(Xd, Td, idx, lr))
         return torch.cat(losses).cpu().numpy()
 
     def predict(self, X) -> np.ndarray:

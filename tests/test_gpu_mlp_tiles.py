@@ -68,3 +68,19 @@ def test_gathered_minibatches_equal_single_steps(n):
     assert np.array_equal(la, lb) and np.array_equal(a.params, b.params) and a.steps == b.steps == 5
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("where", ["numpy", "cuda"])
+def test_row_numbers_out_of_range_are_refused(where):
+    """(The kernel reads row 0 for them: nothing is trained on a wrong row.)"""
+    import torch
+    rows = 40
+    net, th, X, T = _net(rows)
+    for bad in (-1, rows, 1 << 40):
+        idx = np.arange(16).reshape(2, 8)
+        idx[1, 3] = bad
+        with pytest.raises(IndexError):
+            net.train_steps(X, T, idx if where == "numpy" else torch.as_tensor(idx, device="cuda"), 1e-3)
+    assert net.steps == 0 and np.array_equal(net.params, th.astype(np.float32))
+    assert net.train_steps(X, T, np.array([[0, rows - 1]]), 1e-3).shape == (1,)
+    net.close()
