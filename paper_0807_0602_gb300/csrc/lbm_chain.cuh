@@ -1,8 +1,9 @@
-// Chained steps (LBM_KERNEL_CHAIN, FP64): many time steps in one launch.  The work items are (step, tile) pairs in step order; the CTAs
-// draw them one by one from a counter.  An item waits only for the tiles of
-// the step before whose nodes it reads or overwrites (its own tile and its
-// neighbours, at most 32: `deps`), so no step waits for the slowest tile of
-// the whole grid, and neither launches nor empty SMs separate the steps.
+// Chained steps (LBM_KERNEL_CHAIN, FP64): many time steps in one launch.  The
+// work items are (step, tile) pairs in step order; the CTAs draw them one by one
+// from a counter.  An item waits only for the tiles of the step before whose
+// nodes it reads or overwrites (its own tile and its neighbours, at most 32:
+// `deps`), so no step waits for the slowest tile of the whole grid, and neither
+// launches nor empty SMs separate the steps.
 //
 // Why it cannot deadlock: an item depends on items with lower numbers only,
 // and a CTA works its items off in ascending order (it draws the next one
@@ -131,7 +132,7 @@ __global__ void __launch_bounds__(2 * W, (kBidirMinBlocks<S, W>)) k_chain_bidir(
                                                                                ChainTiles ct, int nsteps, int parity,
                                                                                int rot, uint32_t* err) {
     chain_run<2 * W>(ct, nsteps, parity, rot, err, [&](int tile, int par, auto ready) {
-        bidir_tile<S, W, G, false, false>(runs, ct.tiles, tile, par, Shape{}, ready);
+        bidir_tile<S, W, G, false>(runs, ct.tiles, tile, par, Shape{}, ready);
     });
 }
 

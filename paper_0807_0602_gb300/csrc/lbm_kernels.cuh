@@ -1132,8 +1132,8 @@ __device__ __forceinline__ void bar_group(int g) {
 
 // One tile of the march.  `ready` is called once per thread after everything
 // that does not depend on the populations has been loaded (the chained launch
-// waits there for the tiles it reads); NC as in ldp.
-template <typename S, int W, bool G, bool NC, bool UNI, typename Ready>
+// waits there for the tiles it reads).
+template <typename S, int W, bool G, bool UNI, typename Ready>
 __device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, const Tile* __restrict__ tiles, int tile,
                                            int parity, const Shape& shape, Ready ready) {
     using C = typename Prec<S>::C;
@@ -1221,7 +1221,7 @@ __device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, con
                 const unsigned bw = (unsigned)(q.rw * pitch), bm = (unsigned)(q.rm * pitch),
                                bp = (unsigned)(q.rp * pitch);
                 C f[2][9];
-                pull_node<S, NC>(src, plane, bw + sc.xc, bw + sc.xm, bw + sc.xp, bm + sc.xc, bp + sc.xc, bm + sc.xm,
+                pull_node<S, false>(src, plane, bw + sc.xc, bw + sc.xm, bw + sc.xp, bm + sc.xc, bp + sc.xc, bm + sc.xm,
                              bm + sc.xp, bp + sc.xm, bp + sc.xp, smask, cx.sh, f);
                 nA = dens9(f[0]);
                 nB = dens9(f[1]);
@@ -1259,7 +1259,7 @@ __device__ __forceinline__ void bidir_tile(const RunDesc* __restrict__ runs, con
         const char *om = o - pitchB, *op = o + pitchB;
         C f[2][9];
         auto at = [&](int q, const char* row, int dx) {
-            return ldp<NC>(reinterpret_cast<const S*>(row + (unsigned long long)planeB * (unsigned)q + dx * (int)sizeof(S)));
+            return *reinterpret_cast<const S*>(row + (unsigned long long)planeB * (unsigned)q + dx * (int)sizeof(S));
         };
 #pragma unroll
         for (int kk = 0; kk < 2; ++kk) {
@@ -1343,7 +1343,7 @@ template <typename S, int W, bool G>
 __global__ void __launch_bounds__(2 * W, (kBidirMinBlocks<S, W>)) k_step_bidir(const RunDesc* __restrict__ runs,
                                                                               const Tile* __restrict__ tiles,
                                                                               int parity) {
-    bidir_tile<S, W, G, false, false>(runs, tiles, blockIdx.x, parity, Shape{}, [] { step_ready(); });
+    bidir_tile<S, W, G, false>(runs, tiles, blockIdx.x, parity, Shape{}, [] { step_ready(); });
 }
 
 // The same for runs of one size, given as parameters.
@@ -1351,7 +1351,7 @@ template <typename S, int W, bool G>
 __global__ void __launch_bounds__(2 * W, (kBidirMinBlocks<S, W>)) k_step_bidir_alike(const RunDesc* __restrict__ runs,
                                                                                     const Tile* __restrict__ tiles,
                                                                                     int parity, Shape shape) {
-    bidir_tile<S, W, G, false, true>(runs, tiles, blockIdx.x, parity, shape, [] { step_ready(); });
+    bidir_tile<S, W, G, true>(runs, tiles, blockIdx.x, parity, shape, [] { step_ready(); });
 }
 
 // ---- two-columns-per-thread variant ---------------------------------------------
@@ -1583,9 +1583,9 @@ __global__ void __launch_bounds__(W, (kPairMinBlocks<S, W>)) k_step_pair(const R
 template <typename S, int W, int TY>
 constexpr int kTileMinBlocks = sizeof(typename Prec<S>::C) == 8 ? 1 : 1024 / (W * TY);   // 64 registers
 
-template <typename S, int W, int TY, bool G, bool NC, typename Ready>
+template <typename S, int W, int TY, bool G, typename Ready>
 __device__ __forceinline__ void node_tile(const RunDesc* __restrict__ runs, const Tile* __restrict__ tiles, int tile,
-                                          int parity, Ready ready) {   // ready, NC: as in bidir_tile
+                                          int parity, Ready ready) {   // ready: as in bidir_tile
     using C = typename Prec<S>::C;
     __shared__ C sd[TY][2][W];   // [tile row][species][tile column]
 
@@ -1620,7 +1620,7 @@ __device__ __forceinline__ void node_tile(const RunDesc* __restrict__ runs, cons
             // offsets from column -2, so that every offset is non-negative
             const unsigned bw = (unsigned)(q.rw * pitch), bm = (unsigned)(q.rm * pitch), bp = (unsigned)(q.rp * pitch);
             const unsigned xo = (unsigned)(x + 2);
-            pull_node<S, NC>(src - 2, plane, bw + xo, bw + (xo - 1), bw + (xo + 1), bm + xo, bp + xo, bm + (xo - 1),
+            pull_node<S, false>(src - 2, plane, bw + xo, bw + (xo - 1), bw + (xo + 1), bm + xo, bp + xo, bm + (xo - 1),
                          bm + (xo + 1), bp + (xo - 1), bp + (xo + 1), m, cx.sh, f);
             nA = dens9(f[0]);
             nB = dens9(f[1]);
@@ -1640,7 +1640,7 @@ template <typename S, int W, int TY, bool G>
 __global__ void __launch_bounds__(W * TY, (kTileMinBlocks<S, W, TY>)) k_step_tile(const RunDesc* __restrict__ runs,
                                                                                 const Tile* __restrict__ tiles,
                                                                                 int parity) {
-    node_tile<S, W, TY, G, false>(runs, tiles, blockIdx.x, parity, [] { step_ready(); });
+    node_tile<S, W, TY, G>(runs, tiles, blockIdx.x, parity, [] { step_ready(); });
 }
 
 // ---- two steps per launch on small grids ----------------------------------------
