@@ -754,11 +754,11 @@ int wave_height(lbm_t* h, int W, int waves) {
 //     of them: 2048 x 130 103 (bidirectional 124, staged march 180), nine
 //     128 x 80 droplets 54 (72, 155); below that (256 x 32: 20.5, chained 26)
 //     the bidirectional march with tiles of two rows.
-// The creation options' tile_w and tile_h do not enter: a tiling chosen for
-// another kernel is slower on the one that suits the size (droplet batches of
-// 1 to 256 runs, this schedule / 128 x 16 on kernel 9 / on kernel 6: one run of
-// 128 x 80 2.3 / 13 / 27, 32 of 192 x 96 20 / 27 / 37, 256 of 256 x 128 272 / 281 / 324;
-// FP64, nine of 128 x 80: 53, kernel 6 341).  lbm_set_tiling and
+// The creation options' tile_w and tile_h do not enter: a tiling says nothing
+// about the kernel that suits the size (droplet batches, this schedule /
+// 128 x 16 on kernel 9 / on kernel 6: one run of 128 x 80 2.3 / 13 / 27, 32 of
+// 192 x 96 20 / 27 / 37, 256 of them 173 / 168 / 209, 256 of 256 x 128
+// 272 / 281 / 324; FP64, nine of 128 x 80: 53, kernel 6 341).  lbm_set_tiling and
 // lbm_set_schedule take a tiling as it is given.
 Sched default_schedule(lbm_t* h) {
     double nodes = 0.0, strip_rows = 0.0;
